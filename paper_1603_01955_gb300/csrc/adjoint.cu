@@ -122,8 +122,6 @@ __device__ __forceinline__ KC<Dual<R>> dual_consts(const AdjConst<R>& k, int whi
     c.sq_4 = Dual<R>(p.sq_4, which == 1 ? k.dsq4_da : R(0));
     c.hfx = Dual<R>(p.hfx, which == 2 ? R(0.5) : R(0));
     c.fx = Dual<R>(p.fx, which == 2 ? R(1) : R(0));
-    c.hfy = Dual<R>(p.hfy, R(0));
-    c.fy = Dual<R>(p.fy, R(0));
     c.A = c.B = c.A316 = c.CA = c.r = c.rc = c.slope = c.sha = c.shd = c.drho_in = c.drho_out = Dual<R>(0.0);
     c.ref0 = Dual<R>(p.ref0, R(0));
     c.sc = c.isc = Dual<R>(1.0);

@@ -189,8 +189,9 @@ template <class L, class S> __device__ __forceinline__ L bc(S s) {
 __device__ __forceinline__ float2 rcp(float2 a) { return make_float2(rcp(a.x), rcp(a.y)); }
 
 // One cascaded collision (Eq. 4 with Eq. 6-9, 12-13), in place on the
-// deviations d relative to R = ref.  MODE_PERIODIC: body force F, constant
-// rates.  MODE_PRESSURE: no force, s_v and s_q from the local Knudsen number
+// deviations d relative to R = ref.  MODE_PERIODIC: body force F along x
+// (F_y = 0, as everywhere in this library: its terms are left out, which
+// changes no result), constant rates.  MODE_PRESSURE: no force, s_v and s_q from the local Knudsen number
 // Kn = Kn_out rho_out / rho (Sec. 3.2) through Eq. 18 and Eq. 21.
 // rho_kn (pressure channel, optional): the density that sets the local
 // Knudsen number when it is not the node's own (the column's centreline).
@@ -251,11 +252,10 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
     L ux, uy;
     if (MODE == MODE_PERIODIC) {
         ux = fma(jx, irho, bc<L>(c.hfx));
-        uy = fma(jy, irho, bc<L>(c.hfy));
     } else {
         ux = mul(jx, irho);
-        uy = mul(jy, irho);
     }
+    uy = mul(jy, irho);
     const L ux2 = mul(ux, ux), uy2 = mul(uy, uy), uxy = mul(ux, uy);
     const L nux = neg(ux), nuy = neg(uy);
     const L ux_2 = mul(k(2.0), ux), uy_2 = mul(k(2.0), uy);
@@ -275,14 +275,15 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
     L t8 = sub(fma(uy_2, kxxy, fma(ux_2, kxyy, fma(uxy, fma(k(3.0), t5u, nkxy), mul(k(1.0 / 9.0), drho)))),
                fma(ux2, kyyf, fma(uy2, kxxf, kxxyy)));
     if (MODE == MODE_PERIODIC) {
-        const L fx = bc<L>(c.fx), fy = bc<L>(c.fy);
+        const L fx = bc<L>(c.fx);
         const L nrho = neg(rho), nrh = mul(k(0.5), nrho);
-        t3 = fma(nrho, fma(fx, ux, mul(fy, uy)), t3);
-        t4 = fma(nrho, fma(fx, ux, mul(fy, nuy)), t4);
-        t5 = fma(nrh, fma(fx, uy, mul(fy, ux)), t5);
-        t6 = fma(nrh, fma(fy, ux2, mul(mul(k(2.0), fx), uxy)), t6);
-        t7 = fma(nrh, fma(fx, uy2, mul(mul(k(2.0), fy), uxy)), t7);
-        t8 = fma(nrho, fma(fx, mul(ux, uy2), mul(fy, mul(uy, ux2))), t8);
+        const L fux = mul(fx, ux);
+        t3 = fma(nrho, fux, t3);
+        t4 = fma(nrho, fux, t4);
+        t5 = fma(nrh, mul(fx, uy), t5);
+        t6 = fma(nrh, mul(mul(k(2.0), fx), uxy), t6);
+        t7 = fma(nrh, mul(fx, uy2), t7);
+        t8 = fma(nrho, mul(fx, mul(ux, uy2)), t8);
     }
     // kernels g3..g8; hp, hm = (3 g3 +- g4) / 2
     const L g3 = prod(bc<L>(c.s3_12), t3);
@@ -314,18 +315,16 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
     d[8] = add(d[8], add(e6, gm));
     if (MODE == MODE_PERIODIC) {
         // source S = T^-1 S^ (Eq. 9-10), T^-1 in closed form as tinv_apply
-        const L fx = bc<L>(c.fx), fy = bc<L>(c.fy), two = k(2.0), qt = k(0.25);
+        const L fx = bc<L>(c.fx), two = k(2.0), qt = k(0.25);
         const L m1 = prod(rho, fx);
-        const L m2 = prod(rho, fy);
-        const L m3 = mul(two, prod(rho, fma(ux, fx, mul(uy, fy))));
-        const L m4 = mul(two, prod(rho, fma(ux, fx, mul(nuy, fy))));
-        const L m5 = prod(rho, fma(ux, fy, mul(uy, fx)));
-        const L m6 = prod(rho, fma(fy, ux2, mul(mul(two, fx), uxy)));
-        const L m7 = prod(rho, fma(fx, uy2, mul(mul(two, fy), uxy)));
-        const L m8 = mul(two, prod(rho, mul(uxy, fma(fx, uy, mul(fy, ux)))));
+        const L m3 = mul(two, prod(rho, mul(ux, fx)));  // = m4
+        const L m5 = prod(rho, mul(uy, fx));
+        const L m6 = prod(rho, mul(mul(two, fx), uxy));
+        const L m7 = prod(rho, mul(fx, uy2));
+        const L m8 = mul(two, prod(rho, mul(uxy, mul(fx, uy))));
         const L cm = fma(k(-2.0), m8, m3);
-        const L b4 = add(cm, m4), e4 = sub(cm, m4);
-        const L a17 = mul(two, sub(m1, m7)), a26 = mul(two, sub(m2, m6));
+        const L b4 = add(cm, m3), e4 = sub(cm, m3);
+        const L a17 = mul(two, sub(m1, m7)), a26 = mul(k(-2.0), m6);
         const L p56 = add(m5, m6), n56 = sub(m6, m5);
         const L p78 = add(m7, m8), n78 = sub(m8, m7);
         d[0] = add(d[0], sub(m8, m3));  // S_0 = m0 - m3 + m8 with m0 = 0
@@ -350,36 +349,44 @@ template <class T> struct Field {
 };
 
 // Pre-collision deviations at one interior node (x in 1..nx-2) of a pressure
-// channel, gathered element by element; used only to rebuild the end columns.
-template <class T, class R>
-__device__ void gather_node(const SweepArgs& a, const KC<R>& c, const Field<T> f, int x, int y, R o[9]) {
-    auto at = [&](int i, int dy, int xx) -> R {
-        const T* p = f.base + i * f.plane + (long long)(y + dy) * a.pitch + a.xoff + xx;
-        return Codec<T>::dec(__ldg(p), c.isc);
-    };
-    const int rt = row_kind(y, a.ny);
+// channel, gathered element by element through at(i, dy, dx), population i of
+// the node at offset (dx, dy); rt: the row's kind.  Used only to rebuild the
+// end columns.
+template <class R, class At>
+__device__ __forceinline__ void gather_node_at(const KC<R>& c, int rt, At at, R (&o)[9]) {
     const R sha = c.sha, shd = c.shd;  // source at x-1; the source at x+1 gets the negative
-    o[0] = at(0, 0, x);
-    o[1] = at(1, 0, x - 1) + sha;
-    o[3] = at(3, 0, x + 1) - sha;
+    o[0] = at(0, 0, 0);
+    o[1] = at(1, 0, -1) + sha;
+    o[3] = at(3, 0, 1) - sha;
     if (rt & ROW_BOTTOM) {
-        o[2] = at(4, 0, x);
-        o[5] = c.r * at(7, 0, x) + c.rc * (at(8, 0, x - 1) + shd);
-        o[6] = c.r * at(8, 0, x) + c.rc * (at(7, 0, x + 1) - shd);
+        o[2] = at(4, 0, 0);
+        o[5] = c.r * at(7, 0, 0) + c.rc * (at(8, 0, -1) + shd);
+        o[6] = c.r * at(8, 0, 0) + c.rc * (at(7, 0, 1) - shd);
     } else {
-        o[2] = at(2, -1, x);
-        o[5] = at(5, -1, x - 1) + shd;
-        o[6] = at(6, -1, x + 1) - shd;
+        o[2] = at(2, -1, 0);
+        o[5] = at(5, -1, -1) + shd;
+        o[6] = at(6, -1, 1) - shd;
     }
     if (rt & ROW_TOP) {
-        o[4] = at(2, 0, x);
-        o[7] = c.r * at(5, 0, x) + c.rc * (at(6, 0, x + 1) - shd);
-        o[8] = c.r * at(6, 0, x) + c.rc * (at(5, 0, x - 1) + shd);
+        o[4] = at(2, 0, 0);
+        o[7] = c.r * at(5, 0, 0) + c.rc * (at(6, 0, 1) - shd);
+        o[8] = c.r * at(6, 0, 0) + c.rc * (at(5, 0, -1) + shd);
     } else {
-        o[4] = at(4, 1, x);
-        o[7] = at(7, 1, x + 1) - shd;
-        o[8] = at(8, 1, x - 1) + shd;
+        o[4] = at(4, 1, 0);
+        o[7] = at(7, 1, 1) - shd;
+        o[8] = at(8, 1, -1) + shd;
     }
+}
+
+// The same from the populations in global memory.
+template <class T, class R>
+__device__ void gather_node(const SweepArgs& a, const KC<R>& c, const Field<T> f, int x, int y, R (&o)[9]) {
+    gather_node_at<R>(c, row_kind(y, a.ny),
+                      [&](int i, int dy, int dx) -> R {
+                          const T* p = f.base + i * f.plane + (long long)(y + dy) * a.pitch + a.xoff + (x + dx);
+                          return Codec<T>::dec(__ldg(p), c.isc);
+                      },
+                      o);
 }
 
 // Pressure column rebuilt by linear extrapolation (reading of Sec. 3.2):
@@ -389,14 +396,13 @@ __device__ void gather_node(const SweepArgs& a, const KC<R>& c, const Field<T> f
 // the velocity is extrapolated linearly, the non-equilibrium part comes from
 // the first interior neighbour (a linear extrapolation of it as well would
 // amplify the shortest x-wavelength threefold and diverge at tau ~ 30).
+// n1, n2: the pre-collision deviations of columns x + d and x + 2d.
 // Output: deviations relative to R(b).
-template <class T, class R>
-__device__ __forceinline__ void rebuild_column(const SweepArgs& a, const KC<R>& c, const Field<T> f, int x, int y,
-                                            bool inlet, R* out) {
+template <class R>
+__device__ __forceinline__ void rebuild_nodes(const KC<R>& c, int x, bool inlet, const R (&n1)[9], const R (&n2)[9],
+                                              R* out) {
     const int dir = inlet ? 1 : -1;
-    R n1[9], n2[9], e1[9], eb[9];
-    gather_node<T, R>(a, c, f, x + dir, y, n1);
-    gather_node<T, R>(a, c, f, x + 2 * dir, y, n2);
+    R e1[9], eb[9];
     R dr1, jx1, jy1, dr2, jx2, jy2;
     macro_dev(n1, dr1, jx1, jy1);
     macro_dev(n2, dr2, jx2, jy2);
@@ -411,6 +417,17 @@ __device__ __forceinline__ void rebuild_column(const SweepArgs& a, const KC<R>& 
     // on the reference, so only the equilibrium carries R(b)
 #pragma unroll
     for (int i = 0; i < 9; ++i) out[i] = eb[i] + (n1[i] - e1[i]);
+}
+
+// The same from the populations in global memory.
+template <class T, class R>
+__device__ __forceinline__ void rebuild_column(const SweepArgs& a, const KC<R>& c, const Field<T> f, int x, int y,
+                                            bool inlet, R* out) {
+    const int dir = inlet ? 1 : -1;
+    R n1[9], n2[9];
+    gather_node<T, R>(a, c, f, x + dir, y, n1);
+    gather_node<T, R>(a, c, f, x + 2 * dir, y, n2);
+    rebuild_nodes<R>(c, x, inlet, n1, n2, out);
 }
 
 }  // namespace clb

@@ -27,8 +27,7 @@ template <typename R> struct KC {
     R s3_12, s8_4;    // s3/12, s8/4
     R sv_4, sq_4;     // constant s_v/4, s_q/4 (body-force channel)
     R A, B, A316, CA; // pressure channel: tau = A/(rho+B); 3/(16A); (pi B2/4) A
-    R hfx, hfy;       // F/2
-    R fx, fy;         // F
+    R hfx, fx;        // F/2, F (along x)
     R r, rc;          // r_b, 1 - r_b
     R ref0, slope;    // deviation reference R(x) = ref0 + slope x
     R sha, shd;       // added to a value pulled from column x-1: -w slope (axis, diagonal)
@@ -50,7 +49,7 @@ struct SweepArgs {
     double rate_A, rate_B;    // pressure channel: tau = A / (rho + B)
     double rate_C;            // pi * B2 / 4
     double r;                 // CBBSR bounce-back fraction (Eq. 20)
-    double gx, gy;            // body force per unit mass (Eq. 9, 13)
+    double gx;                // body force per unit mass, along x (Eq. 9, 13)
     // Stored values are deviations f - w_i R(x) from a reference density
     // R(x) = ref0 + ref_slope * x (R = 0 for FP64 storage).
     double ref0, ref_slope;

@@ -530,7 +530,6 @@ SweepArgs make_args(const clb_sim* s) {
     a.rate_C = kPi * s->b2 / 4.0;
     a.r = s->r;
     a.gx = s->drive == CLB_DRIVE_BODY_FORCE ? s->g : 0.0;
-    a.gy = 0.0;
     a.ref0 = s->ref0;
     a.ref_slope = s->ref_slope;
     a.drho_in = s->rho_in - s->ref_at(0);

@@ -353,9 +353,7 @@ template <typename R> static void fill(KC<R>& c, const SweepArgs& a) {
     c.A316 = a.rate_A > 0 ? R(3.0 / (16.0 * a.rate_A)) : R(0);
     c.CA = R(a.rate_C * a.rate_A);
     c.hfx = R(0.5 * a.gx);
-    c.hfy = R(0.5 * a.gy);
     c.fx = R(a.gx);
-    c.fy = R(a.gy);
     c.r = R(a.r);
     c.rc = R(1.0 - a.r);
     c.ref0 = R(a.ref0);
