@@ -114,4 +114,22 @@ cudaError_t launch_sweep_tma(int storage, int mode, int variant, const SweepArgs
                              unsigned* sched, unsigned* status);
 int tma_variant_count();
 
+// Several steps per launch of a small channel held in shared memory (tile.cu).
+struct TilePlan {
+    int h = 0;            // steps per launch at most (0: no plan)
+    bool whole = false;   // one block holds the whole channel (no halo)
+    bool pack = false;    // two nodes per packed FP32 collision
+    bool big = false;     // the larger constant plane in shared memory
+    int cs = 0;           // elements between columns in shared memory
+    int cpp = 0;          // columns (pack: pairs) per pass of the block's threads
+    int main = 0;         // threads that step columns; the rest step a pressure channel's ends
+    int threads = 0, blocks = 0;
+    size_t smem = 0;
+};
+constexpr int kTileMaxSteps = 4096;  // steps per launch of a whole channel in one block
+TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_cap);
+// Allow the plan's shared memory on the current device.
+cudaError_t tile_opt_in(int storage, int mode, const TilePlan& p);
+cudaError_t launch_tiles(int storage, int mode, const TilePlan& p, const SweepArgs& a, int nsteps, cudaStream_t st);
+
 }  // namespace clb

@@ -86,6 +86,7 @@ struct clb_sim {
     int withhold_tile = -1; // testing: TMA tile withheld in the first launch
     int graph_steps = 0;    // sweeps per replayed CUDA graph (0: no replay); even
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // per parity of `cur` at the chunk start
+    TilePlan tile;          // several steps per launch (tile.h > 0): small channels, default engine
     int kn_mode = 0;        // 1: centreline Knudsen number (pressure channel)
     void* rc = nullptr;     // centreline densities: [2 sides][2 rows][rc_stride], compute type
     int rc_stride = 0;
@@ -705,6 +706,19 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
         s->pipeline = 1;  // small channels: the direct sweep has the shorter latency per step
     else
         s->pipeline = (o.storage == CLB_FP32_SHIFTED) ? 2 : 3;
+    // small channels of the default engine: several steps per launch
+    if (o.pipeline == 0 && o.vec == 0 && o.block_x == 0 && s->pipeline == 1 && o.test_withhold_tile < 0) {
+        const int mode = drive == CLB_DRIVE_PRESSURE ? MODE_PRESSURE : MODE_PERIODIC;
+        int dev = 0, sms = 0, cap = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        s->tile = plan_tiles(o.storage, mode, nx, ny, sms, (size_t)std::max(cap, 0));
+        if (s->tile.h > 0 && tile_opt_in(o.storage, mode, s->tile) != cudaSuccess) {
+            cudaGetLastError();
+            s->tile = TilePlan{};
+        }
+    }
     {
         // graph replay: not with the testing option
         int k = 0;
@@ -712,6 +726,8 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
             k = o.graph_steps;
         else if (o.graph_steps == 0)
             k = ((long long)nx * ny < (1LL << 20)) ? 64 : 0;
+        // whole launches of a tiled channel in a chunk by default
+        if (o.graph_steps == 0 && s->tile.h > 0 && !s->tile.whole) k = 2 * s->tile.h * std::max(1, 32 / s->tile.h);
         if (o.test_withhold_tile >= 0) k = 0;
         s->graph_steps = k + (k & 1);  // even: a chunk ends on the buffer it started from
     }
@@ -810,26 +826,47 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
     return CLB_OK;
 }
 
-// One sweep launch from buffer `cur` (direct or TMA engine).
-static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur) {
+// One launch from buffer `cur`: a sweep (direct or TMA engine), or `steps`
+// steps of the channel in tiles.
+static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur, int steps = 1) {
     const size_t rc_side = (size_t)2 * s->rc_stride * (s->storage == CLB_FP64 ? 8 : 4);
     a.fin = s->buf[cur];
     a.fout = s->buf[cur ^ 1];
     a.rc_in = static_cast<const char*>(s->rc) + cur * rc_side;
     a.rc_out = static_cast<char*>(s->rc) + (cur ^ 1) * rc_side;
     a.tile_order = cur;  // alternate the TMA sweep's tile order with the buffers
+    if (s->tile.h > 0) return launch_tiles(s->storage, mode, s->tile, a, steps, s->stream);
     return s->pipeline >= 2 ? launch_sweep_tma(s->storage, mode, s->pipeline - 2, a, s->stream, s->sched, s->status)
                             : launch_sweep(s->storage, mode, s->vec, s->block_x, a, s->stream);
 }
 
-// Capture graph_steps consecutive sweeps starting from buffer `cur` into an
+// Queue n steps from buffer *cur as launches of about equal length, each of at
+// most the steps the engine takes at once; `even`: an even number of launches,
+// so that they end on the buffer they started from.  *done counts the steps queued.
+static cudaError_t launch_steps(clb_sim* s, SweepArgs& a, int mode, int* cur, int64_t n, bool even, int64_t* done) {
+    const int64_t most = s->tile.h > 0 ? s->tile.h : 1;
+    int64_t launches = (n + most - 1) / most;
+    if (even && launches % 2) ++launches;
+    *done = 0;
+    for (; launches > 0; --launches) {
+        const int64_t k = (n - *done + launches - 1) / launches;
+        cudaError_t e = launch_single(s, a, mode, *cur, (int)k);
+        if (e != cudaSuccess) return e;
+        *cur ^= 1;
+        *done += k;
+        s->withhold_tile = a.withhold_tile = -1;
+    }
+    return cudaSuccess;
+}
+
+// Capture graph_steps consecutive steps starting from buffer `cur` into an
 // executable graph (programmatic launch edges are kept).
 static cudaError_t build_graph(clb_sim* s, const SweepArgs& base, int mode, int cur, cudaGraphExec_t* out) {
     SweepArgs a = base;
     cudaError_t e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return e;
-    cudaError_t le = cudaSuccess;
-    for (int k = 0; k < s->graph_steps && le == cudaSuccess; ++k, cur ^= 1) le = launch_single(s, a, mode, cur);
+    int64_t done = 0;
+    cudaError_t le = launch_steps(s, a, mode, &cur, s->graph_steps, true, &done);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(s->stream, &g);
     if (le != cudaSuccess || e != cudaSuccess) {
@@ -847,8 +884,9 @@ clb_status clb_step(clb_sim* s, int64_t n) {
     if (n < 0) return fail(CLB_EINVAL, "clb_step: n < 0");
     const int mode = s->drive == CLB_DRIVE_PRESSURE ? MODE_PRESSURE : MODE_PERIODIC;
     SweepArgs a = make_args(s);
-    // replayed chunks (the chunk length is even, so `cur` is where it started)
-    for (; s->graph_steps > 0 && n >= s->graph_steps; n -= s->graph_steps) {
+    // replayed chunks (of an even number of launches, so `cur` is where it
+    // started); a channel that one block holds takes them as one launch each
+    for (; s->graph_steps > 0 && !s->tile.whole && n >= s->graph_steps; n -= s->graph_steps) {
         if (!s->graph[s->cur]) {
             cudaError_t e = build_graph(s, a, mode, s->cur, &s->graph[s->cur]);
             if (e != cudaSuccess) return fail(CLB_ECUDA, "clb_step: capturing the sweep graph: %s", cudaGetErrorString(e));
@@ -857,13 +895,10 @@ clb_status clb_step(clb_sim* s, int64_t n) {
         if (e != cudaSuccess) return fail(CLB_ECUDA, "clb_step: graph launch: %s", cudaGetErrorString(e));
         s->step += s->graph_steps;
     }
-    for (int64_t t = 0; t < n; ++t) {
-        cudaError_t e = launch_single(s, a, mode, s->cur);
-        if (e != cudaSuccess) return fail(CLB_ECUDA, "clb_step: sweep launch: %s", cudaGetErrorString(e));
-        s->cur ^= 1;
-        ++s->step;
-        s->withhold_tile = a.withhold_tile = -1;
-    }
+    int64_t done = 0;
+    const cudaError_t e = launch_steps(s, a, mode, &s->cur, n, false, &done);
+    s->step += done;
+    if (e != cudaSuccess) return fail(CLB_ECUDA, "clb_step: sweep launch: %s", cudaGetErrorString(e));
     return CLB_OK;
 }
 
