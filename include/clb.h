@@ -321,15 +321,19 @@ typedef struct clb_adjoint clb_adjoint; /* opaque */
 /* Run the forward pass, keeping a checkpoint every checkpoint_every steps
  * (<= 0: ceil(sqrt(nsteps))), and return J.  opts->storage CLB_FP64 or
  * CLB_FP32_SHIFTED (states and adjoints in that precision; the parameter
- * sums are FP64).  r < 0 takes r_b from Eq. 21 with opts->sigma (the gradient
- * is still with respect to r_b).  Device memory: (ceil(nsteps/C) + C + 5)
- * states of 9 nx ny elements.  Synchronises.  nx * ny <= 2^22.
+ * sums are FP64, or FP32 pairs of 48 bits).  r < 0 takes r_b from Eq. 21 with
+ * opts->sigma (the gradient is still with respect to r_b).  Device memory:
+ * (ceil(nsteps/C) + C + 4) states of 9 nx ny elements; for FP32 grids of at most
+ * 512 nodes (ceil(nsteps/C) + 2 C + 3) states and 16 C nx elements, or with C
+ * in the place of 2 C where the allocator refuses that.  Synchronises.
+ * nx * ny <= 2^22.
  * Engine: a grid whose two states fit in one block's shared memory
  * (2 * 9 nx ny elements <= about 200 KB: 2800 nodes in FP32) runs the
  * forward pass as one launch of one block and each backward pass as one
- * launch of an 8-block cluster; larger grids, or opts->pipeline = 1, use one
- * launch per step.  Both give the same states; the FP64 sums of J and of the
- * gradient are taken in different orders. */
+ * launch of a thread-block cluster (a pair of blocks for the FP32 grids above,
+ * else 8 or 16); larger grids, or opts->pipeline = 1, use one launch per step.
+ * All give the same states; the sums of J and of the gradient are taken in
+ * different orders. */
 clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, double g, int64_t nsteps,
                                int checkpoint_every, const clb_opts* opts, clb_adjoint** out, double* J);
 

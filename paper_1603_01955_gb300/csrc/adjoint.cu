@@ -8,11 +8,11 @@
 // (Eq. 5, periodic x, walls Eq. 20), C collides every node (Eq. 4, 6-13).  The
 // adjoint runs backwards: mu = J_C(P f_t)^T lambda_{t+1} per node, then
 // lambda_t = P^T mu, while r_b, a and G collect lambda_{t+1}^T dC/dtheta and
-// mu^T dP/dr.  J_C^T lambda is formed column by column with forward-mode dual
-// numbers pushed through the very collision template the sweeps use (one
-// tangent per input population, one for a, one for G); P^T is written out by
-// hand as a gather (each post-collision population is pulled by one node, or
-// by two wall nodes).  The forward keeps a checkpoint every C steps (C ~
+// mu^T dP/dr.  J_C^T lambda is the collision's reverse, written out by hand
+// (reverse_collide): the moments and kernels of the forward step, then their
+// adjoints in the opposite order, which also yield the terms of s_v, s_q and G.
+// P^T is a gather (each post-collision population is pulled by one node, or by
+// two wall nodes).  The forward keeps a checkpoint every C steps (C ~
 // sqrt(N)) and recomputes each segment before walking it backwards.
 // Parameter sums are FP64; states and adjoints are FP32 or FP64.
 #include <cuda_runtime.h>
@@ -20,39 +20,12 @@
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/clb.h"
 #include "clb_device.cuh"
 #include "clb_internal.h"
-
-namespace clb {
-
-// Forward-mode dual number with one tangent component.
-template <class R> struct Dual {
-    R v, d;
-    __host__ __device__ Dual() : v(0), d(0) {}
-    __host__ __device__ Dual(double x) : v(R(x)), d(0) {}
-    __host__ __device__ Dual(R x, R dx) : v(x), d(dx) {}
-};
-template <class R> __device__ __forceinline__ Dual<R> operator+(Dual<R> a, Dual<R> b) { return {a.v + b.v, a.d + b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a, Dual<R> b) { return {a.v - b.v, a.d - b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a) { return {-a.v, -a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator*(Dual<R> a, Dual<R> b) {
-    return {a.v * b.v, a.v * b.d + a.d * b.v};
-}
-template <class R> __device__ __forceinline__ Dual<R> operator/(Dual<R> a, Dual<R> b) {
-    const R q = a.v / b.v;
-    return {q, (a.d - q * b.d) / b.v};
-}
-template <class R> __device__ __forceinline__ Dual<R>& operator+=(Dual<R>& a, Dual<R> b) { return a = a + b; }
-template <class R> __device__ __forceinline__ Dual<R>& operator-=(Dual<R>& a, Dual<R> b) { return a = a - b; }
-template <class R> __device__ __forceinline__ Dual<R> rcp(Dual<R> a) {
-    const R q = R(1) / a.v;
-    return {q, -a.d * q * q};
-}
-
-}  // namespace clb
 
 using namespace clb;
 
@@ -68,64 +41,139 @@ template <class R> struct AdjConst {
     int nx, ny;
 };
 
-// The 9 pre-collision populations of node (x, y): pull with periodic x and
-// the CBBSR walls (Eq. 20 and its mirror), from a state [9][ny][nx].
-template <class R>
-__device__ __forceinline__ void pull(const R* f, int nx, int ny, int x, int y, R r, R rc, R (&o)[9]) {
-    const int nn = nx * ny;
-    const int xm = x == 0 ? nx - 1 : x - 1;
-    const int xp = x == nx - 1 ? 0 : x + 1;
-    auto at = [&](int i, int yy, int xx) -> R { return f[i * nn + yy * nx + xx]; };
-    o[0] = at(0, y, x);
-    o[1] = at(1, y, xm);
-    o[3] = at(3, y, xp);
-    if (y == 0) {
-        o[2] = at(4, 0, x);
-        o[5] = r * at(7, 0, x) + rc * at(8, 0, xm);
-        o[6] = r * at(8, 0, x) + rc * at(7, 0, xp);
-    } else {
-        o[2] = at(2, y - 1, x);
-        o[5] = at(5, y - 1, xm);
-        o[6] = at(6, y - 1, xp);
-    }
-    if (y == ny - 1) {
-        o[4] = at(2, y, x);
-        o[7] = r * at(5, y, x) + rc * at(6, y, xp);
-        o[8] = r * at(6, y, x) + rc * at(5, y, xm);
-    } else {
-        o[4] = at(4, y + 1, x);
-        o[7] = at(7, y + 1, xp);
-        o[8] = at(8, y + 1, xm);
-    }
-}
-
 template <class R>
 __global__ void adj_forward_kernel(const R* fin, R* fout, AdjConst<R> k) {
     const int nn = k.nx * k.ny;
     for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x) {
         R d[9];
-        pull(fin, k.nx, k.ny, node % k.nx, node / k.nx, k.r, k.rc, d);
+        gather_at(fin, pull_of(k.nx, k.ny, node % k.nx, node / k.nx), k.r, k.rc, d);
         collide<R, MODE_PERIODIC>(d, k.ref, k.c);
         for (int i = 0; i < 9; ++i) fout[i * nn + node] = d[i];
     }
 }
 
-// Collision constants with the tangent of one parameter: which = 0 none,
-// 1 a (through s_v and s_q), 2 G.
+// A sum over many steps: FP64 as it is, FP32 terms in a pair of FP32 numbers
+// (the rounding errors of the running sum, exact by Knuth's two-sum, go to the
+// second), 48 bits without the FP64 pipe.
+template <class R> struct Acc {
+    R s = 0;
+    __device__ __forceinline__ void add(R v) { s += v; }
+    __device__ __forceinline__ void add(R a, R b) { s += a * b; }  // a b
+    __device__ __forceinline__ double value() const { return (double)s; }
+};
+template <> struct Acc<float> {
+    float s = 0, e = 0;
+    __device__ __forceinline__ void add(float v) {
+        const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)));
+        s = t;
+    }
+    __device__ __forceinline__ void add(float a, float b) {
+        const float v = __fmul_rn(a, b);
+        e = __fadd_rn(e, __fmaf_rn(a, b, -v));
+        add(v);
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
+// The sums of one thread: l . dC/d(s_v/4), dC/d(s_q/4), dC/dG, and mu . dP/dr.
+template <class R> struct ParamSums {
+    Acc<R> sv, sq, g, r;
+};
+
+// m = J_C(d)^T l for one node of a body-force channel (collide, MODE_PERIODIC)
+// and the node's parameter terms.  Capital names are adjoints.
 template <class R>
-__device__ __forceinline__ KC<Dual<R>> dual_consts(const AdjConst<R>& k, int which) {
-    KC<Dual<R>> c;
-    const KC<R>& p = k.c;
-    c.s3_12 = Dual<R>(p.s3_12, R(0));
-    c.s8_4 = Dual<R>(p.s8_4, R(0));
-    c.sv_4 = Dual<R>(p.sv_4, which == 1 ? k.dsv4_da : R(0));
-    c.sq_4 = Dual<R>(p.sq_4, which == 1 ? k.dsq4_da : R(0));
-    c.hfx = Dual<R>(p.hfx, which == 2 ? R(0.5) : R(0));
-    c.fx = Dual<R>(p.fx, which == 2 ? R(1) : R(0));
-    c.A = c.B = c.A316 = c.CA = c.r = c.rc = c.slope = c.sha = c.shd = c.drho_in = c.drho_out = Dual<R>(0.0);
-    c.ref0 = Dual<R>(p.ref0, R(0));
-    c.sc = c.isc = Dual<R>(1.0);
-    return c;
+__device__ __forceinline__ void reverse_collide(const R (&d)[9], const R (&l)[9], R ref, const KC<R>& c, R (&m)[9],
+                                                ParamSums<R>& sum) {
+    const R h = R(0.5), q = R(0.25), two = R(2), third = R(1.0 / 3.0);
+    // forward: moments, braces and kernels
+    const R a57 = d[5] + d[7], a68 = d[6] + d[8], p57 = d[5] - d[7], p86 = d[8] - d[6];
+    const R nkxy = a68 - a57, kxxyy = a57 + a68, kxxy = p57 - p86, kxyy = p57 + p86;
+    const R s13 = d[1] + d[3], s24 = d[2] + d[4];
+    const R kxx = s13 + kxxyy, kyy = s24 + kxxyy, drho = d[0] + s13 + s24 + kxxyy;
+    const R jx = d[1] - d[3] + kxyy, jy = d[2] - d[4] + kxxy;
+    const R rho = ref + drho, irho = rcp(rho), fx = c.fx;
+    const R ux = jx * irho + c.hfx, uy = jy * irho;
+    const R kx = kxx + third * ref, ky = kyy + third * ref;
+    const R ux2 = ux * ux, uy2 = uy * uy, uxy = ux * uy, rf = rho * fx;
+    const R t5u = rho * uxy + nkxy;
+    const R t3 = rho * (ux2 + uy2) + R(2.0 / 3.0) * drho - (kxx + kyy) - rf * ux;
+    const R t4 = rho * (ux2 - uy2) + (kyy - kxx) - rf * ux;
+    const R t5 = t5u - h * rf * uy;
+    const R t6 = two * ux * t5u - uy * kx + kxxy - rf * uxy;
+    const R t7 = two * uy * t5u - ux * ky + kxyy - h * rf * uy2;
+    const R g3 = c.s3_12 * t3, g4 = c.sv_4 * t4, g5 = c.sv_4 * t5;
+    const R hp = R(1.5) * g3 + h * g4, hm = R(1.5) * g3 - h * g4;
+    const R g6 = c.sq_4 * t6 - uy * hp - two * ux * g5;
+    const R g7 = c.sq_4 * t7 - ux * hm - two * uy * g5;
+    // reverse of Eq. 6 and of the source (Eq. 9-10)
+    const R A1 = l[1] + l[3], A2 = l[2] + l[4], D1 = l[1] - l[3], D2 = l[2] - l[4];
+    const R S5 = l[5] + l[7], S6 = l[6] + l[8], E5 = l[7] - l[5], E6 = l[8] - l[6];
+    const R A = A1 + A2, S = S5 + S6;
+    const R G8 = R(4) * l[0] - two * A + S;
+    const R M1 = h * D1, M3 = h * A1 - l[0], M5 = q * (S5 - S6), M6 = -(h * D2 + q * (E5 + E6));
+    const R M7 = q * (E6 - E5) - h * D1, M8 = l[0] - h * A + q * S;
+    // g8 .. g3
+    const R G7 = two * D1 + E5 - E6 - two * ux * G8;
+    const R G6 = two * D2 + E5 + E6 - two * uy * G8;
+    const R HP = -(uy2 * G8 + uy * G6), HM = -(ux2 * G8 + ux * G7);
+    const R G5 = S5 - S6 - R(4) * uxy * G8 - two * (uy * G7 + ux * G6);
+    const R G4 = A1 - A2 + h * (HP - HM);
+    const R G3 = two * S - R(4) * l[0] - A - two * G8 + R(1.5) * (HP + HM);
+    R UXY = R(-4) * g5 * G8;
+    R UX = -(two * (ux * hm + g7) * G8 + hm * G7 + two * g5 * G6);
+    R UY = -(two * (uy * hp + g6) * G8 + hp * G6 + two * g5 * G7);
+    const R T8 = c.s8_4 * G8, T7 = c.sq_4 * G7, T6 = c.sq_4 * G6, T5 = c.sv_4 * G5, T4 = c.sv_4 * G4, T3 = c.s3_12 * G3;
+    sum.sv.add(t4, G4);
+    sum.sv.add(t5, G5);
+    sum.sq.add(t6, G6);
+    sum.sq.add(t7, G7);
+    // the braces of Eq. 7 and the source's moments: the force terms first, as
+    // one factor of rho G and its own adjoint
+    const R uxy2 = ux * uy2;
+    const R T34 = T3 + T4;
+    // d/d(rho fx) of every force term
+    const R RF = -(T34 * ux + h * T5 * uy + T6 * uxy + h * T7 * uy2 + T8 * uxy2) + M1 + two * M3 * ux + M5 * uy +
+                 two * M6 * uxy + M7 * uy2 + two * M8 * uxy2;
+    const R FU = -T34 + two * M3 + (two * M8 - T8) * uy2;              // rf * d/dux (but uxy)
+    const R FV = M5 - h * T5 + (two * M7 - T7) * uy + (R(4) * M8 - two * T8) * uxy;  // rf * d/duy (but uxy)
+    const R T5U = T5 + two * (uy * T7 + ux * T6) + R(3) * uxy * T8;
+    UXY += (R(3) * t5u + nkxy) * T8 + rho * T5U + rf * (two * M6 - T6);
+    UX += two * (kxyy - ux * ky) * T8 - ky * T7 + two * t5u * T6 + two * rho * ux * T34 + rf * FU + uy * UXY;
+    UY += two * (kxxy - uy * kx) * T8 + two * t5u * T7 - kx * T6 + two * rho * uy * (T3 - T4) + rf * FV + ux * UXY;
+    sum.g.add(rho * RF + h * UX);  // u_x holds G/2 as well
+    R DR = fx * RF + (ux2 + uy2) * T3 + (ux2 - uy2) * T4 + uxy * T5U;  // through rho
+    const R JX = irho * UX, JY = irho * UY;
+    DR -= irho * (jx * JX + jy * JY);
+    DR += R(2.0 / 3.0) * T3 + R(1.0 / 9.0) * T8;
+    const R KXX = -(uy2 * T8 + uy * T6 + T4 + T3), KYY = T4 - T3 - ux2 * T8 - ux * T7;
+    const R NKXY = uxy * T8 + T5U;
+    const R KXXY = two * uy * T8 + T6 + JY, KXYY = two * ux * T8 + T7 + JX;
+    const R X13 = KXX + DR, X24 = KYY + DR, KT = KXX + KYY + DR - T8;
+    m[0] = l[0] + DR;
+    m[1] = l[1] + (X13 + JX);
+    m[3] = l[3] + (X13 - JX);
+    m[2] = l[2] + (X24 + JY);
+    m[4] = l[4] + (X24 - JY);
+    const R K57 = KT - NKXY, K68 = KT + NKXY, P57 = KXXY + KXYY, P86 = KXYY - KXXY;
+    m[5] = l[5] + (K57 + P57);
+    m[7] = l[7] + (K57 - P57);
+    m[6] = l[6] + (K68 - P86);
+    m[8] = l[8] + (K68 + P86);
+}
+
+// mu . dP/dr of a wall node: f5, f6 (bottom) or f7, f8 (top) of the pull
+// r A + (1 - r) B collect mu (A - B) (Eq. 20).
+template <class R> __device__ __forceinline__ void wall_term(R mu, R a, R b, Acc<R>& s) {
+    if constexpr (std::is_same<R, float>::value) {
+        const float v = __fsub_rn(a, b), z = __fsub_rn(v, a);  // a - b and its rounding error
+        const float e = __fsub_rn(__fsub_rn(a, __fsub_rn(v, z)), __fadd_rn(b, z));
+        s.add(mu, v);
+        s.add(mu, e);
+    } else {
+        s.add(mu, a - b);
+    }
 }
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
@@ -142,58 +190,95 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 constexpr int kAdjThreads = 128;
 
-// mu = J_C^T lambda_{t+1} at every node (indexed like the pre-collision
-// populations), and the parameter terms of step t added to this block's slots
-// acc[k * gridDim.x + blockIdx.x], k = 0, 1, 2 (r, a, G).  Each slot has one
-// writer and the launches run in stream order, so every slot is summed in a
-// fixed order and the gradient is the same bit for bit on every run.
+// lambda_t(node) = (P^T mu)(node): each post-collision population of step t is
+// pulled by the node it streams to, or, at a wall, by the bounce-back and the
+// specular terms of Eq. 20 (two nodes of the wall row).  The offsets and
+// weights for one node, as Pull for the forward direction.
+__device__ __forceinline__ Pull push_of(int nx, int ny, int x, int y) {
+    Pull p;
+    const int nn = nx * ny;
+    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+    auto at = [&](int i, int yy, int xx) { return i * nn + yy * nx + xx; };
+    p.top = y == ny - 1;
+    p.bottom = y == 0;
+    p.wb[0] = p.wb[1] = p.wt[0] = p.wt[1] = 0;
+    p.o[0] = at(0, y, x);
+    p.o[1] = at(1, y, xp);  // f1 at x is pulled by x+1
+    p.o[3] = at(3, y, xm);
+    // moving up (2, 5, 6): pulled by row y+1, or by the top-wall terms
+    p.o[2] = p.top ? at(4, y, x) : at(2, y + 1, x);
+    p.o[5] = p.top ? at(7, y, x) : at(5, y + 1, xp);
+    p.o[6] = p.top ? at(8, y, x) : at(6, y + 1, xm);
+    if (p.top) {
+        p.wt[0] = at(8, y, xp);
+        p.wt[1] = at(7, y, xm);
+    }
+    // moving down (4, 7, 8): pulled by row y-1, or by the bottom-wall terms
+    p.o[4] = p.bottom ? at(2, y, x) : at(4, y - 1, x);
+    p.o[7] = p.bottom ? at(5, y, x) : at(7, y - 1, xm);
+    p.o[8] = p.bottom ? at(6, y, x) : at(8, y - 1, xp);
+    if (p.bottom) {
+        p.wb[0] = at(6, y, xm);
+        p.wb[1] = at(5, y, xp);
+    }
+    return p;
+}
+template <class R>
+__device__ __forceinline__ void transpose_at(const R* mu, const Pull& p, R r, R rc, R (&o)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) o[i] = mu[p.o[i]];
+    if (p.top) {
+        o[5] = r * o[5] + rc * mu[p.wt[0]];
+        o[6] = r * o[6] + rc * mu[p.wt[1]];
+    }
+    if (p.bottom) {
+        o[7] = r * o[7] + rc * mu[p.wb[0]];
+        o[8] = r * o[8] + rc * mu[p.wb[1]];
+    }
+}
+
+// One node's share of backward step t: lambda_{t+1} from mu_{t+1} (or given,
+// at the last step), mu_t = J_C^T lambda, the parameter terms.  f: the state
+// at t; all [9][ny][nx].
+template <class R>
+__device__ __forceinline__ void back_node(const R* f, const R* mu_next, const R* lam, R* mu, int node, int x, int y,
+                                          const AdjConst<R>& k, ParamSums<R>& sum) {
+    const int nn = k.nx * k.ny;
+    const Pull p = pull_of(k.nx, k.ny, x, y);
+    R fb[9], l[9], m[9];
+    gather_at(f, p, k.r, k.rc, fb);
+    if (mu_next)
+        transpose_at(mu_next, push_of(k.nx, k.ny, x, y), k.r, k.rc, l);
+    else
+        for (int i = 0; i < 9; ++i) l[i] = lam[i * nn + node];
+    reverse_collide(fb, l, k.ref, k.c, m, sum);
+    for (int i = 0; i < 9; ++i) mu[i * nn + node] = m[i];
+    if (p.bottom) {
+        wall_term(m[5], f[p.o[5]], f[p.wb[0]], sum.r);
+        wall_term(m[6], f[p.o[6]], f[p.wb[1]], sum.r);
+    }
+    if (p.top) {
+        wall_term(m[7], f[p.o[7]], f[p.wt[0]], sum.r);
+        wall_term(m[8], f[p.o[8]], f[p.wt[1]], sum.r);
+    }
+}
+
+// mu_t at every node from mu_{t+1}, and the parameter terms of step t added to
+// this block's slots acc[k * gridDim.x + blockIdx.x], k = 0, 1, 2 (r, a, G).
+// Each slot has one writer and the launches run in stream order, so every slot
+// is summed in a fixed order and the gradient is the same bit for bit on every
+// run.
 template <class R>
 __global__ void __launch_bounds__(kAdjThreads)
-    adj_back_kernel(const R* f_t, const R* lam, R* mu, double* acc, AdjConst<R> k) {
+    adj_back_kernel(const R* f_t, const R* mu_next, const R* lam, R* mu, double* acc, AdjConst<R> k) {
     __shared__ double sh[kAdjThreads];
     const int nn = k.nx * k.ny;
-    double gr = 0, ga = 0, gg = 0;
-    for (int base = blockIdx.x * blockDim.x; base < nn; base += gridDim.x * blockDim.x) {
-        const int node = base + threadIdx.x;
-        if (node < nn) {
-            const int x = node % k.nx, y = node / k.nx;
-            R fb[9], l[9];
-            pull(f_t, k.nx, k.ny, x, y, k.r, k.rc, fb);
-            for (int i = 0; i < 9; ++i) l[i] = lam[i * nn + node];
-            const KC<Dual<R>> c0 = dual_consts(k, 0);
-            R m[9];
-            for (int j = 0; j < 9; ++j) {  // column j of the collision Jacobian
-                Dual<R> d[9];
-                for (int i = 0; i < 9; ++i) d[i] = Dual<R>(fb[i], i == j ? R(1) : R(0));
-                collide<Dual<R>, MODE_PERIODIC>(d, Dual<R>(k.ref, R(0)), c0);
-                R s = 0;
-                for (int i = 0; i < 9; ++i) s += l[i] * d[i].d;
-                m[j] = s;
-                mu[j * nn + node] = s;
-            }
-            for (int which = 1; which <= 2; ++which) {  // dC/da, dC/dG
-                const KC<Dual<R>> cp = dual_consts(k, which);
-                Dual<R> d[9];
-                for (int i = 0; i < 9; ++i) d[i] = Dual<R>(fb[i], R(0));
-                collide<Dual<R>, MODE_PERIODIC>(d, Dual<R>(k.ref, R(0)), cp);
-                double s = 0;
-                for (int i = 0; i < 9; ++i) s += (double)l[i] * (double)d[i].d;
-                if (which == 1)
-                    ga += s;
-                else
-                    gg += s;
-            }
-            // dP/dr at the wall rows (Eq. 20): d fbar5/dr = f7(x) - f8(x-1), ...
-            const int xm = x == 0 ? k.nx - 1 : x - 1;
-            const int xp = x == k.nx - 1 ? 0 : x + 1;
-            auto at = [&](int i, int xx) -> double { return (double)f_t[i * nn + y * k.nx + xx]; };
-            if (y == 0) gr += (double)m[5] * (at(7, x) - at(8, xm)) + (double)m[6] * (at(8, x) - at(7, xp));
-            if (y == k.ny - 1) gr += (double)m[7] * (at(5, x) - at(6, xp)) + (double)m[8] * (at(6, x) - at(5, xm));
-        }
-    }
-    gr = block_sum(gr, sh);
-    ga = block_sum(ga, sh);
-    gg = block_sum(gg, sh);
+    ParamSums<R> sum;
+    for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x)
+        back_node(f_t, mu_next, lam, mu, node, node % k.nx, node / k.nx, k, sum);
+    const double gr = block_sum(sum.r.value(), sh);
+    const double ga = block_sum(sum.sv.value() * (double)k.dsv4_da + sum.sq.value() * (double)k.dsq4_da, sh);
+    const double gg = block_sum(sum.g.value(), sh);
     if (threadIdx.x == 0) {
         acc[0 * gridDim.x + blockIdx.x] += gr;
         acc[1 * gridDim.x + blockIdx.x] += ga;
@@ -201,90 +286,61 @@ __global__ void __launch_bounds__(kAdjThreads)
     }
 }
 
-// lambda_t = P^T mu: each post-collision population of step t is pulled by
-// the node it streams to, or, at a wall, by the bounce-back and the specular
-// terms of Eq. 20 (two nodes of the wall row).
+// One node's term of J = (1/nx) sum u_x of the final post-collision state, and
+// its lambda_N = dJ/df_N: u_x = sum_i e_ix f_i / rho - G/2, so
+// dJ/df_i = (e_ix - u_x - G/2) / (nx rho).
 template <class R>
-__global__ void adj_transpose_kernel(const R* mu, R* lam, AdjConst<R> k) {
-    const int nx = k.nx, ny = k.ny, nn = nx * ny;
-    for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x) {
-        const int x = node % nx, y = node / nx;
-        const int xm = x == 0 ? nx - 1 : x - 1;
-        const int xp = x == nx - 1 ? 0 : x + 1;
-        auto M = [&](int i, int yy, int xx) -> R { return mu[i * nn + yy * nx + xx]; };
-        R o[9];
-        o[0] = M(0, y, x);
-        o[1] = M(1, y, xp);  // f1 at x is pulled by x+1
-        o[3] = M(3, y, xm);
-        // moving up (2, 5, 6): pulled by row y+1, or by the top-wall terms
-        if (y == ny - 1) {
-            o[2] = M(4, y, x);
-            o[5] = k.r * M(7, y, x) + k.rc * M(8, y, xp);
-            o[6] = k.r * M(8, y, x) + k.rc * M(7, y, xm);
-        } else {
-            o[2] = M(2, y + 1, x);
-            o[5] = M(5, y + 1, xp);
-            o[6] = M(6, y + 1, xm);
-        }
-        // moving down (4, 7, 8): pulled by row y-1, or by the bottom-wall terms
-        if (y == 0) {
-            o[4] = M(2, 0, x);
-            o[7] = k.r * M(5, 0, x) + k.rc * M(6, 0, xm);
-            o[8] = k.r * M(6, 0, x) + k.rc * M(5, 0, xp);
-        } else {
-            o[4] = M(4, y - 1, x);
-            o[7] = M(7, y - 1, xm);
-            o[8] = M(8, y - 1, xp);
-        }
-        for (int i = 0; i < 9; ++i) lam[i * nn + node] = o[i];
+__device__ __forceinline__ double flow_term(const R* f, R* lam, int node, const AdjConst<R>& k) {
+    const int nn = k.nx * k.ny;
+    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+    double rho = (double)k.ref, jx = 0;
+    for (int i = 0; i < 9; ++i) {
+        const double v = (double)f[i * nn + node];
+        rho += v;
+        jx += ex[i] * v;
     }
+    const double ux = jx / rho - 0.5 * (double)k.c.fx;
+    for (int i = 0; i < 9; ++i) lam[i * nn + node] = R((ex[i] - ux - 0.5 * (double)k.c.fx) / (k.nx * rho));
+    return ux / k.nx;
 }
 
-// J = (1/nx) sum u_x of the final post-collision state and lambda_N = dJ/df_N:
-// u_x = sum_i e_ix f_i / rho - G/2, so dJ/df_i = (e_ix - u_x - G/2) / (nx rho).
 template <class R>
 __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* lam, double* acc, AdjConst<R> k) {
     __shared__ double sh[kAdjThreads];
     const int nn = k.nx * k.ny;
-    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
     double js = 0;
-    for (int base = blockIdx.x * blockDim.x; base < nn; base += gridDim.x * blockDim.x) {
-        const int node = base + threadIdx.x;
-        if (node < nn) {
-            double rho = (double)k.ref, jx = 0;
-            for (int i = 0; i < 9; ++i) {
-                const double v = (double)f[i * nn + node];
-                rho += v;
-                jx += ex[i] * v;
-            }
-            const double ux = jx / rho - 0.5 * (double)k.c.fx;
-            js += ux / k.nx;
-            for (int i = 0; i < 9; ++i) lam[i * nn + node] = R((ex[i] - ux - 0.5 * (double)k.c.fx) / (k.nx * rho));
-        }
-    }
+    for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x)
+        js += flow_term(f, lam, node, k);
     js = block_sum(js, sh);
     if (threadIdx.x == 0) acc[3 * gridDim.x + blockIdx.x] = js;
 }
 
 // ------------------------------------------------------ resident engine
 //
-// For a grid whose two states fit in one block's shared memory, the whole
-// checkpointed forward pass is one launch of one block, with block barriers
-// between the steps; the backward walk over every segment is one launch of a
-// thread-block cluster, with cluster barriers between its phases (the
-// arithmetic is that of the kernels above).  In the backward step the 9 + 2
-// forward-mode columns of each node's collision are spread over separate
-// threads.  The parameter sums stay per thread (FP64, in step order) and are
-// added by fixed trees at the end, so the gradient is the same bit for bit on
-// every run.
-constexpr int kResThreads = 256;  // the dual-number collision needs ~160-250 registers
-constexpr int kCols = 11;         // 9 population tangents, then a and G
+// The whole checkpointed forward pass is one launch, of one block with block
+// barriers between the steps where two states fit in its shared memory, else
+// (FP32) of a thread-block cluster with cluster barriers; the backward walk
+// over every segment is one launch of a cluster.  The parameter sums stay per thread (in step
+// order) and are added by fixed trees at the end, so the gradient is the same
+// bit for bit on every run.
+//
+// Backward, FP32 grids of at most one node per thread of a block: a pair of
+// blocks (adj_pair_backward_kernel).  One recomputes a segment's steps while
+// the other walks the segment after it backwards, each with its state in shared
+// memory and block barriers only; the cluster barrier separates segments.
+// Other grids: every block of the cluster takes its share of the nodes of each
+// step, with a cluster barrier between steps (adj_cl_backward_kernel).
+// 4 x 64 nodes, FP32, per step: forward 0.36 us, backward 0.94 us (0.63 and
+// 6.46 us with the pulls worked out every step and J_C^T lambda formed by eleven
+// forward-mode columns over 16 blocks); both are bound by issue and latency in
+// their one block.  20 x 128 nodes, backward by a cluster: 3.2 us (31.4 us).
+constexpr int kResThreads = 512;
 
 __device__ __forceinline__ double res_block_sum(double v, double* sh) {
     sh[threadIdx.x] = v;
     __syncthreads();
     for (int w = kResThreads / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+        if ((int)threadIdx.x < w && threadIdx.x + w < blockDim.x) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
     }
     const double r = sh[0];
@@ -292,25 +348,35 @@ __device__ __forceinline__ double res_block_sum(double v, double* sh) {
     return r;
 }
 
-// One step of the whole grid in shared memory, a -> b (and optionally to a
-// global copy `out`).
-template <class R>
-__device__ __forceinline__ void res_step(const R* a, R* b, R* out, const AdjConst<R>& k) {
-    const int nn = k.nx * k.ny;
-    for (int node = threadIdx.x; node < nn; node += kResThreads) {
-        R d[9];
-        pull(a, k.nx, k.ny, node % k.nx, node / k.nx, k.r, k.rc, d);
-        collide<R, MODE_PERIODIC>(d, k.ref, k.c);
-        for (int i = 0; i < 9; ++i) {
-            b[i * nn + node] = d[i];
-            if (out) out[i * nn + node] = d[i];
+// Steps of the whole grid in shared memory, from copy s to copy o (then the
+// other way round), with the block's barrier after each.  ONE: at most one
+// node per thread, whose pull is worked out once.  Before each collision,
+// visit(node, pulled populations, pull, state) sees the node.
+template <bool ONE, class R, class V>
+__device__ __forceinline__ void res_steps(R*& s, R*& o, long long nsteps, const AdjConst<R>& k, V&& visit) {
+    const int nn = k.nx * k.ny, node1 = threadIdx.x;
+    Pull p1{};
+    if (ONE && node1 < nn) p1 = pull_of(k.nx, k.ny, node1 % k.nx, node1 / k.nx);
+    for (long long t = 0; t < nsteps; ++t) {
+        for (int node = node1; node < nn; node += ONE ? nn : blockDim.x) {
+            const Pull p = ONE ? p1 : pull_of(k.nx, k.ny, node % k.nx, node / k.nx);
+            R d[9];
+            gather_at(s, p, k.r, k.rc, d);
+            visit(t, node, d, p, s);
+            collide<R, MODE_PERIODIC>(d, k.ref, k.c);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) o[i * nn + node] = d[i];
         }
+        __syncthreads();
+        R* q = s;
+        s = o;
+        o = q;
     }
 }
 
 // Forward pass from f^eq(rho_out, 0): checkpoint s (the state at step s C)
 // into ckpt + s state_elems, then J and lambda_N (as adj_final_kernel).
-template <class R>
+template <class R, bool ONE>
 __global__ void __launch_bounds__(kResThreads)
     adj_res_forward_kernel(R* ckpt, size_t state_elems, int every, long long nsteps, R* lam_final, double* J,
                            AdjConst<R> k) {
@@ -319,46 +385,19 @@ __global__ void __launch_bounds__(kResThreads)
     R* a = reinterpret_cast<R*>(sm_raw);
     R* b = a + n9;
     double* red = reinterpret_cast<double*>(sm_raw + ((2 * n9 * sizeof(R) + 15) / 16) * 16);
-    for (int e = threadIdx.x; e < n9; e += kResThreads) a[e] = R(0);  // zero deviations
+    for (int e = threadIdx.x; e < n9; e += blockDim.x) a[e] = R(0);  // zero deviations
     __syncthreads();
-    for (long long t = 0; t < nsteps; ++t) {
-        if (t % every == 0) {
-            R* c = ckpt + (size_t)(t / every) * state_elems;
-            for (int e = threadIdx.x; e < n9; e += kResThreads) c[e] = a[e];
-        }
-        res_step<R>(a, b, nullptr, k);
-        __syncthreads();
-        R* t2 = a;
-        a = b;
-        b = t2;
+    for (long long t = 0; t < nsteps; t += every) {
+        R* c = ckpt + (size_t)(t / every) * state_elems;
+        for (int e = threadIdx.x; e < n9; e += blockDim.x) c[e] = a[e];
+        res_steps<ONE>(a, b, min((long long)every, nsteps - t), k, [](long long, int, const R*, const Pull&, const R*) {});
     }
-    const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
     double js = 0;
-    for (int node = threadIdx.x; node < nn; node += kResThreads) {
-        double rho = (double)k.ref, jx = 0;
-        for (int i = 0; i < 9; ++i) {
-            const double v = (double)a[i * nn + node];
-            rho += v;
-            jx += ex[i] * v;
-        }
-        const double ux = jx / rho - 0.5 * (double)k.c.fx;
-        js += ux / k.nx;
-        for (int i = 0; i < 9; ++i) lam_final[i * nn + node] = R((ex[i] - ux - 0.5 * (double)k.c.fx) / (k.nx * rho));
-    }
+    for (int node = threadIdx.x; node < nn; node += blockDim.x) js += flow_term(a, lam_final, node, k);
     js = res_block_sum(js, red);
     if (threadIdx.x == 0) *J = js;
 }
 
-// The backward walk over every segment, spread over one thread-block cluster
-// of `gridDim.x` blocks: recompute the segment's states from its checkpoint,
-// then per step mu_t = J_C^T lambda_{t+1}, one thread per node and column,
-// with lambda_{t+1} = P^T mu_{t+1} gathered on the fly from the previous
-// step's mu (lambda_N itself for the first step), so one cluster barrier
-// separates the steps.  mu (two buffers) and the segment states are in global
-// memory (a few KB each, resident in L2); the cluster barrier (release /
-// acquire at cluster scope) orders them.  Every block runs the same loop
-// counts, so every barrier is reached by all of them.  Each block's
-// parameter sums go to part[rank * 3 + 0..2], added on the host in rank order.
 constexpr int kClusterMax = 16;
 
 __device__ __forceinline__ void cluster_barrier() {
@@ -372,46 +411,217 @@ __device__ __forceinline__ int cluster_rank() {
     return (int)r;
 }
 
-// lambda_t(node) = (P^T mu)(node): each post-collision population of step t is
-// pulled by the node it streams to, or, at a wall, by the bounce-back and the
-// specular terms of Eq. 20 (as adj_transpose_kernel).
 template <class R>
-__device__ __forceinline__ void transpose_at(const R* mu, int nx, int ny, int x, int y, R r, R rc, R (&o)[9]) {
-    const int nn = nx * ny;
-    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-    auto M = [&](int i, int yy, int xx) -> R { return mu[i * nn + yy * nx + xx]; };
-    o[0] = M(0, y, x);
-    o[1] = M(1, y, xp);
-    o[3] = M(3, y, xm);
-    if (y == ny - 1) {
-        o[2] = M(4, y, x);
-        o[5] = r * M(7, y, x) + rc * M(8, y, xp);
-        o[6] = r * M(8, y, x) + rc * M(7, y, xm);
-    } else {
-        o[2] = M(2, y + 1, x);
-        o[5] = M(5, y + 1, xp);
-        o[6] = M(6, y + 1, xm);
-    }
-    if (y == 0) {
-        o[4] = M(2, 0, x);
-        o[7] = r * M(5, 0, x) + rc * M(6, 0, xm);
-        o[8] = r * M(6, 0, x) + rc * M(5, 0, xp);
-    } else {
-        o[4] = M(4, y - 1, x);
-        o[7] = M(7, y - 1, xm);
-        o[8] = M(8, y - 1, xp);
+__device__ __forceinline__ void write_sums(const ParamSums<R>& sum, const AdjConst<R>& k, double* red, double* out) {
+    const double gr = res_block_sum(sum.r.value(), red);
+    const double ga = res_block_sum(sum.sv.value() * (double)k.dsv4_da + sum.sq.value() * (double)k.dsq4_da, red);
+    const double gg = res_block_sum(sum.g.value(), red);
+    if (threadIdx.x == 0) {
+        out[0] = gr;
+        out[1] = ga;
+        out[2] = gg;
     }
 }
 
+// The backward walk by a pair of blocks (see above): per step of a segment,
+// `seg` holds the pulled populations of every node, coalesced, and the eight
+// values each column's wall terms differ by (pair_elems elements).  bufs: the
+// segments it holds, 2 (recomputation of one beside the walk over the other) or
+// 1 (in turn).  Nodes <= threads of a block.
+__host__ __device__ constexpr size_t pair_elems(int nx, int ny) { return 9 * (size_t)nx * ny + 8 * (size_t)nx; }
+
+template <class R>
+__global__ void __launch_bounds__(kResThreads)
+    adj_pair_backward_kernel(const R* ckpt, R* seg, size_t state_elems, int every, long long nsteps, int bufs,
+                             const R* lam_final, double* part, AdjConst<R> k) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ double red[kResThreads];
+    const int nx = k.nx, ny = k.ny, nn = nx * ny, n9 = 9 * nn;
+    R* a = reinterpret_cast<R*>(sm_raw);
+    R* b = a + n9;
+    const int rank = cluster_rank();
+    const int node = threadIdx.x;
+    const bool live = node < nn;
+    const int x = live ? node % nx : 0, y = live ? node / nx : 0;
+    const bool bottom = live && y == 0, top = live && y == ny - 1;
+    const long long nseg = (nsteps + every - 1) / every;
+    const size_t step_elems = pair_elems(nx, ny), seg_elems = step_elems * every;
+    auto length = [&](long long s) { return (int)min((long long)every, nsteps - s * every); };
+
+    auto recompute = [&](long long s) {
+        const R* c = ckpt + (size_t)s * state_elems;
+        for (int e = threadIdx.x; e < n9; e += blockDim.x) a[e] = c[e];
+        __syncthreads();
+        R* out = seg + (size_t)(s % bufs) * seg_elems;
+        res_steps<true>(a, b, length(s), k, [&](long long t, int n1, const R* d, const Pull& p, const R* f) {
+            R* w = out + (size_t)t * step_elems;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) w[i * nn + n1] = d[i];
+            R* e = w + n9 + x;
+            if (bottom) {
+                e[0] = f[p.o[5]];
+                e[nx] = f[p.wb[0]];
+                e[2 * nx] = f[p.o[6]];
+                e[3 * nx] = f[p.wb[1]];
+            }
+            if (top) {
+                e[4 * nx] = f[p.o[7]];
+                e[5 * nx] = f[p.wt[0]];
+                e[6 * nx] = f[p.o[8]];
+                e[7 * nx] = f[p.wt[1]];
+            }
+        });
+    };
+
+    ParamSums<R> sum;
+    Pull p{};
+    if (live) p = push_of(nx, ny, x, y);
+    auto walk = [&](long long s) {
+        const R* in = seg + (size_t)(s % bufs) * seg_elems;
+        const int len = length(s);
+        struct Step {
+            R fb[9], w[8];
+        };
+        auto load = [&](int j, Step& v) {
+            const R* q = in + (size_t)j * step_elems;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v.fb[i] = q[i * nn + node];
+            const R* e = q + n9 + x;
+            if (bottom)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v.w[i] = e[i * nx];
+            if (top)
+#pragma unroll
+                for (int i = 4; i < 8; ++i) v.w[i] = e[i * nx];
+        };
+        Step cur, nxt;
+        if (live) load(len - 1, cur);
+        for (int j = len - 1; j >= 0; --j) {
+            if (live) {
+                R l[9], m[9];
+                if (s == nseg - 1 && j == len - 1)
+                    for (int i = 0; i < 9; ++i) l[i] = lam_final[i * nn + node];
+                else
+                    transpose_at(a, p, k.r, k.rc, l);
+                if (j > 0) load(j - 1, nxt);  // the next step's values arrive meanwhile
+                reverse_collide(cur.fb, l, k.ref, k.c, m, sum);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) b[i * nn + node] = m[i];
+                if (bottom) {
+                    wall_term(m[5], cur.w[0], cur.w[1], sum.r);
+                    wall_term(m[6], cur.w[2], cur.w[3], sum.r);
+                }
+                if (top) {
+                    wall_term(m[7], cur.w[4], cur.w[5], sum.r);
+                    wall_term(m[8], cur.w[6], cur.w[7], sum.r);
+                }
+                cur = nxt;
+            }
+            __syncthreads();
+            R* q = a;
+            a = b;
+            b = q;
+        }
+    };
+
+    // block 1 recomputes, block 0 walks; every barrier is reached by both
+    if (bufs == 2) {
+        if (rank == 1) recompute(nseg - 1);
+        cluster_barrier();
+        for (long long s = nseg - 1; s >= 0; --s) {
+            if (rank == 1) {
+                if (s > 0) recompute(s - 1);
+            } else {
+                walk(s);
+            }
+            cluster_barrier();
+        }
+    } else {
+        for (long long s = nseg - 1; s >= 0; --s) {
+            if (rank == 1) recompute(s);
+            cluster_barrier();
+            if (rank == 0) walk(s);
+            cluster_barrier();
+        }
+    }
+    if (rank == 0) write_sums(sum, k, red, part);
+}
+
+// One block's nodes of a cluster, dealt out by whole warps, one to each block
+// in turn: the FP64 pipe takes 64 cycles per warp and instruction however few
+// lanes are live, so the fewest warps per SM finish first.  each(node, x, y);
+// a block's threads cover its share in one round (ONE) or several.
+struct ClusterNodes {
+    int first, step, nx, x, y;
+    __device__ ClusterNodes(int rank, int nx_) : nx(nx_) {
+        first = (((int)threadIdx.x >> 5) * (int)gridDim.x + rank) * 32 + ((int)threadIdx.x & 31);
+        step = (int)(gridDim.x * blockDim.x);
+        y = first / nx;
+        x = first - y * nx;
+    }
+    template <class F> __device__ __forceinline__ void each(int nn, F&& f) const {
+        if (first < nn) f(first, x, y);
+        for (int node = first + step; node < nn; node += step) f(node, node % nx, node / nx);
+    }
+};
+
+// The forward pass by a cluster, states (two, in `work`) in global memory: a
+// few hundred KB, resident in L2.  J's sums per block go to part[rank].
+template <class R>
+__global__ void __launch_bounds__(kResThreads)
+    adj_cl_forward_kernel(R* ckpt, R* work, size_t state_elems, int every, long long nsteps, R* lam_final,
+                          double* part, AdjConst<R> k) {
+    __shared__ double red[kResThreads];
+    const int nn = k.nx * k.ny, rank = cluster_rank();
+    const ClusterNodes mine(rank, k.nx);
+    R* a = work;
+    R* b = work + state_elems;
+    mine.each(nn, [&](int node, int, int) {  // zero deviations
+        for (int i = 0; i < 9; ++i) a[i * nn + node] = ckpt[i * nn + node] = R(0);
+    });
+    cluster_barrier();
+    for (long long t = 0; t < nsteps; ++t) {
+        R* c = (t + 1) % every == 0 && t + 1 < nsteps ? ckpt + (size_t)((t + 1) / every) * state_elems : nullptr;
+        mine.each(nn, [&](int node, int x, int y) {
+            R d[9];
+            gather_at(a, pull_of(k.nx, k.ny, x, y), k.r, k.rc, d);
+            collide<R, MODE_PERIODIC>(d, k.ref, k.c);
+            for (int i = 0; i < 9; ++i) {
+                b[i * nn + node] = d[i];
+                if (c) c[i * nn + node] = d[i];
+            }
+        });
+        cluster_barrier();
+        R* q = a;
+        a = b;
+        b = q;
+    }
+    double js = 0;
+    mine.each(nn, [&](int node, int, int) { js += flow_term(a, lam_final, node, k); });
+    js = res_block_sum(js, red);
+    if (threadIdx.x == 0) part[rank] = js;
+}
+
+// The backward walk by a cluster of `gridDim.x` blocks: recompute the
+// segment's states from its checkpoint, then per step mu_t = J_C^T lambda_{t+1}
+// with lambda_{t+1} = P^T mu_{t+1} gathered on the fly from the previous
+// step's mu (lambda_N itself for the first step), so one cluster barrier
+// separates the steps.  mu (two buffers) and the segment states are in global
+// memory (resident in L2); the cluster barrier (release / acquire at cluster
+// scope) orders them.  Every block runs
+// the same loop counts, so every barrier is reached by all of them.  Each
+// block's parameter sums go to part[rank * 3 + 0..2], added on the host in rank
+// order.
 template <class R>
 __global__ void __launch_bounds__(kResThreads)
     adj_cl_backward_kernel(const R* ckpt, R* seg, size_t state_elems, int every, long long nsteps,
                            const R* lam_final, R* mu0, R* mu1, double* part, AdjConst<R> k) {
     __shared__ double red[kResThreads];
-    const int nn = k.nx * k.ny, n9 = 9 * nn, nx = k.nx, ny = k.ny;
+    const int nn = k.nx * k.ny, n9 = 9 * nn;
     const int rank = cluster_rank();
-    const int g0 = rank * kResThreads + (int)threadIdx.x, gs = (int)gridDim.x * kResThreads;
-    double gr = 0, ga = 0, gg = 0;
+    const int e0 = rank * (int)blockDim.x + (int)threadIdx.x, es = (int)(gridDim.x * blockDim.x);
+    const ClusterNodes mine(rank, k.nx);
+    ParamSums<R> sum;
     const R* mu_next = nullptr;  // mu of step t + 1 (none before the first backward step)
     R* mu_cur = mu0;
     const long long nseg = (nsteps + every - 1) / every;
@@ -419,76 +629,51 @@ __global__ void __launch_bounds__(kResThreads)
         const long long t0 = s * every;
         const int len = (int)min((long long)every, nsteps - t0);
         const R* c = ckpt + (size_t)s * state_elems;
-        for (int e = g0; e < n9; e += gs) seg[e] = c[e];
+        for (int e = e0; e < n9; e += es) seg[e] = c[e];
         cluster_barrier();
         for (int j = 1; j < len; ++j) {  // recompute the segment's states
             const R* a = seg + (size_t)(j - 1) * state_elems;
             R* b = seg + (size_t)j * state_elems;
-            for (int node = g0; node < nn; node += gs) {
+            mine.each(nn, [&](int node, int x, int y) {
                 R d[9];
-                pull(a, nx, ny, node % nx, node / nx, k.r, k.rc, d);
+                gather_at(a, pull_of(k.nx, k.ny, x, y), k.r, k.rc, d);
                 collide<R, MODE_PERIODIC>(d, k.ref, k.c);
                 for (int i = 0; i < 9; ++i) b[i * nn + node] = d[i];
-            }
+            });
             cluster_barrier();
         }
         for (int j = len - 1; j >= 0; --j) {
             const R* ft = seg + (size_t)j * state_elems;
-            for (int it = g0; it < nn * kCols; it += gs) {
-                const int node = it / kCols, col = it - node * kCols;
-                const int x = node % nx, y = node / nx;
-                R lam[9];
-                if (mu_next) {
-                    transpose_at(mu_next, nx, ny, x, y, k.r, k.rc, lam);
-                } else {
-                    for (int i = 0; i < 9; ++i) lam[i] = lam_final[i * nn + node];
-                }
-                R fb[9];
-                pull(ft, nx, ny, x, y, k.r, k.rc, fb);
-                const KC<Dual<R>> cd = dual_consts(k, col < 9 ? 0 : col - 8);
-                Dual<R> d[9];
-                for (int i = 0; i < 9; ++i) d[i] = Dual<R>(fb[i], i == col ? R(1) : R(0));
-                collide<Dual<R>, MODE_PERIODIC>(d, Dual<R>(k.ref, R(0)), cd);
-                if (col < 9) {
-                    R m = 0;
-                    for (int i = 0; i < 9; ++i) m += lam[i] * d[i].d;
-                    mu_cur[col * nn + node] = m;
-                    // dP/dr at the wall rows (Eq. 20)
-                    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-                    auto at = [&](int i, int xx) -> double { return (double)ft[i * nn + y * nx + xx]; };
-                    if (y == 0 && col == 5) gr += (double)m * (at(7, x) - at(8, xm));
-                    if (y == 0 && col == 6) gr += (double)m * (at(8, x) - at(7, xp));
-                    if (y == ny - 1 && col == 7) gr += (double)m * (at(5, x) - at(6, xp));
-                    if (y == ny - 1 && col == 8) gr += (double)m * (at(6, x) - at(5, xm));
-                } else {
-                    double sum = 0;
-                    for (int i = 0; i < 9; ++i) sum += (double)lam[i] * (double)d[i].d;
-                    if (col == 9)
-                        ga += sum;
-                    else
-                        gg += sum;
-                }
-            }
+            mine.each(nn, [&](int node, int x, int y) {
+                back_node(ft, mu_next, lam_final, mu_cur, node, x, y, k, sum);
+            });
             cluster_barrier();
             mu_next = mu_cur;
             mu_cur = mu_cur == mu0 ? mu1 : mu0;
         }
     }
-    gr = res_block_sum(gr, red);
-    ga = res_block_sum(ga, red);
-    gg = res_block_sum(gg, red);
-    if (threadIdx.x == 0) {
-        part[rank * 3 + 0] = gr;
-        part[rank * 3 + 1] = ga;
-        part[rank * 3 + 2] = gg;
-    }
+    write_sums(sum, k, red, part + rank * 3);
 }
 
 // Shared memory of the resident forward kernel: two states and the block sum.
 size_t res_smem(int nx, int ny, size_t elem) {
     return ((2 * 9 * (size_t)nx * ny * elem + 15) / 16) * 16 + kResThreads * sizeof(double);
 }
+// Threads of a resident block: one node each, by whole warps.
+int res_threads(int nx, int ny) { return std::min(kResThreads, (nx * ny + 31) / 32 * 32); }
 constexpr size_t kResSmemCap = 200 * 1024;
+// Largest FP32 grid of the cluster kernels, whose 16 blocks cost 0.3 us per
+// thousand nodes and step beyond 8192; one launch per step costs 5 us forward
+// and 12 us backward whatever the grid.  Measured, us per step forward +
+// backward, cluster / launches: 100 x 50 2.3 + 3.8 / 4.8 + 12.3; 160 x 100
+// 3.9 + 7.0 / 5.2 + 12.4; 200 x 160 6.1 + 11.6 / 6.1 + 12.6; 320 x 200
+// 9.6 + 20.9 / 5.8 + 14.6.
+constexpr int kClusterNodes = 24576;
+// Nodes up to which the forward pass of a resident grid stays in one block.
+// FP32: 10 x 100 1.5 us per step there, 15 x 100 2.1, 20 x 128 3.3 (cluster 1.7).
+// FP64, bound by the FP64 pipe: 4 x 64 12.4 us there, 6.5 us in a cluster (one
+// warp per SM), where 4 x 32 takes as long.
+int block_nodes(size_t elem) { return elem == 8 ? 128 : 1024; }
 
 }  // namespace
 
@@ -500,13 +685,15 @@ struct clb_adjoint {
     void* ckpt = nullptr;  // checkpoints: state at steps 0, C, 2C, ...
     int nckpt = 0;
     void* seg = nullptr;   // one recomputed segment: C + 1 states
-    void* lam[2] = {nullptr, nullptr};
+    void* mu0 = nullptr;   // mu of one backward step, mu of the next
     void* lam_final = nullptr;  // lambda_N = dJ/df_N, kept for every backward call
     void* mu = nullptr;
     double* acc = nullptr; // per-block partial sums [4][nb]: r, a, G and J
     int nb = 0;            // blocks of every adjoint launch
     bool resident = false; // resident engine: the forward pass in one block, the backward in one cluster
-    int cluster = 0;       // blocks of the backward cluster (0: not yet launched)
+    bool pair = false;     // ... the backward in a pair of blocks; seg then holds seg_bufs segments of pulled steps
+    int seg_bufs = 1;
+    int cluster = 0;       // blocks of the backward cluster otherwise (0: not yet launched)
     AdjConst<float> kf;
     AdjConst<double> kd;
     double J = 0;
@@ -562,38 +749,23 @@ cudaError_t sum_partials(clb_adjoint* h, int rows, double* out) {
     return cudaSuccess;
 }
 
-template <class R> cudaError_t set_res_smem(size_t bytes) {
-    return cudaFuncSetAttribute(adj_res_forward_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+template <class K> cudaError_t set_res_smem(K kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// Both passes in one block each (resident engine).
-template <class R> cudaError_t forward_resident(clb_adjoint* h) {
-    const size_t smem = res_smem(h->nx, h->ny, sizeof(R));
-    cudaError_t e = set_res_smem<R>(smem);
-    if (e != cudaSuccess) return e;
-    adj_res_forward_kernel<R><<<1, kResThreads, smem, h->stream>>>(
-        static_cast<R*>(h->ckpt), h->state_elems, h->every, (long long)h->nsteps, static_cast<R*>(h->lam_final),
-        h->acc, kconst<R>(h));
-    e = cudaGetLastError();
-    double J = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&J, h->acc, sizeof J, cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e == cudaSuccess) h->J = J;
-    return e;
-}
-
-// Launch the cluster backward kernel with `cl` blocks (16 needs the
-// non-portable cluster size, which the device may refuse).
-template <class R> cudaError_t launch_cl_backward(clb_adjoint* h, int cl) {
-    auto kern = adj_cl_backward_kernel<R>;
+// Launch fn's kernel with its arguments as one cluster of `cl` blocks (more
+// than 8 need the non-portable cluster size, which the device may refuse).
+template <class K, class... A>
+cudaError_t launch_cluster(K kern, int cl, int threads, size_t smem, cudaStream_t st, A... args) {
     if (cl > 8) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(kResThreads);
-    cfg.stream = h->stream;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cl;
@@ -601,27 +773,81 @@ template <class R> cudaError_t launch_cl_backward(clb_adjoint* h, int cl) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<const R*>(h->ckpt), static_cast<R*>(h->seg), h->state_elems,
-                              h->every, (long long)h->nsteps, static_cast<const R*>(h->lam_final),
-                              static_cast<R*>(h->lam[0]), static_cast<R*>(h->mu), h->acc, kconst<R>(h));
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// Threads per block of a cluster of cl blocks: a node each, as far as they go.
+int cl_threads(const clb_adjoint* h, int cl) {
+    const int warps = (h->nx * h->ny + 31) / 32;
+    return std::min(kResThreads, 32 * std::max(1, (warps + cl - 1) / cl));
+}
+
+// Run launch(cl) with the largest cluster the device takes (16 blocks, else
+// the portable 8).
+template <class F> cudaError_t with_cluster(clb_adjoint* h, F&& launch) {
+    if (h->cluster) return launch(h->cluster);
+    h->cluster = kClusterMax;
+    cudaError_t e = launch(h->cluster);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        h->cluster = 8;
+        e = launch(h->cluster);
+    }
+    if (e != cudaSuccess) h->cluster = 0;
+    return e;
+}
+
+// The forward pass in one block, or in one cluster (resident engine).
+template <class R> cudaError_t forward_resident(clb_adjoint* h) {
+    const size_t smem = res_smem(h->nx, h->ny, sizeof(R));
+    int sums = 1;
+    cudaError_t e;
+    if (smem <= kResSmemCap && h->nx * h->ny <= block_nodes(sizeof(R))) {
+        auto kern = h->nx * h->ny <= kResThreads ? adj_res_forward_kernel<R, true> : adj_res_forward_kernel<R, false>;
+        e = set_res_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        kern<<<1, res_threads(h->nx, h->ny), smem, h->stream>>>(
+            static_cast<R*>(h->ckpt), h->state_elems, h->every, (long long)h->nsteps, static_cast<R*>(h->lam_final),
+            h->acc, kconst<R>(h));
+        e = cudaGetLastError();
+    } else {
+        e = with_cluster(h, [&](int cl) {
+            return launch_cluster(adj_cl_forward_kernel<R>, cl, cl_threads(h, cl), 0, h->stream,
+                                  static_cast<R*>(h->ckpt), static_cast<R*>(h->seg), h->state_elems, h->every,
+                                  (long long)h->nsteps, static_cast<R*>(h->lam_final), h->acc, kconst<R>(h));
+        });
+        sums = h->cluster;
+    }
+    double part[kClusterMax] = {};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(part, h->acc, sums * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return e;
+    h->J = 0;
+    for (int r = 0; r < sums; ++r) h->J += part[r];  // rank order
+    return cudaSuccess;
+}
+
+template <class R> cudaError_t launch_cl_backward(clb_adjoint* h, int cl) {
+    return launch_cluster(adj_cl_backward_kernel<R>, cl, cl_threads(h, cl), 0, h->stream, static_cast<const R*>(h->ckpt),
+                          static_cast<R*>(h->seg), h->state_elems, h->every, (long long)h->nsteps,
+                          static_cast<const R*>(h->lam_final), static_cast<R*>(h->mu0), static_cast<R*>(h->mu),
+                          h->acc, kconst<R>(h));
+}
+
+cudaError_t launch_pair_backward(clb_adjoint* h) {
+    using R = float;
+    const size_t smem = 2 * h->state_elems * sizeof(R);
+    cudaError_t e = set_res_smem(adj_pair_backward_kernel<R>, smem);
+    if (e != cudaSuccess) return e;
+    return launch_cluster(adj_pair_backward_kernel<R>, 2, res_threads(h->nx, h->ny), smem, h->stream,
+                          static_cast<const R*>(h->ckpt), static_cast<R*>(h->seg), h->state_elems, h->every,
+                          (long long)h->nsteps, h->seg_bufs, static_cast<const R*>(h->lam_final), h->acc, kconst<R>(h));
 }
 
 template <class R> cudaError_t backward_resident(clb_adjoint* h, double* out3) {
-    // the largest cluster the device runs (16 blocks, else the portable 8)
-    int cl = h->cluster;
-    cudaError_t e = cudaSuccess;
-    if (cl == 0) {
-        cl = kClusterMax;
-        e = launch_cl_backward<R>(h, cl);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            cl = 8;
-            e = launch_cl_backward<R>(h, cl);
-        }
-        if (e == cudaSuccess) h->cluster = cl;
-    } else {
-        e = launch_cl_backward<R>(h, cl);
-    }
+    cudaError_t e = h->pair ? launch_pair_backward(h)
+                            : with_cluster(h, [&](int cl) { return launch_cl_backward<R>(h, cl); });
+    const int cl = h->pair ? 1 : h->cluster;  // blocks with sums
     double part[3 * kClusterMax];
     if (e == cudaSuccess) e = cudaMemcpyAsync(part, h->acc, 3 * cl * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -676,11 +902,8 @@ template <class R> cudaError_t backward_run(clb_adjoint* h, double seed, double 
     const AdjConst<R>& k = kconst<R>(h);
     const int nb = h->nb;
     cudaError_t e = cudaMemsetAsync(h->acc, 0, (size_t)3 * nb * sizeof(double), h->stream);
-    R* lam = static_cast<R*>(h->lam[0]);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(lam, h->lam_final, h->state_elems * sizeof(R), cudaMemcpyDeviceToDevice, h->stream);
-    R* lam2 = static_cast<R*>(h->lam[1]);
-    R* mu = static_cast<R*>(h->mu);
+    const R* mu_next = nullptr;
+    R* mu = static_cast<R*>(h->mu0);
     for (int64_t s = (h->nsteps - 1) / h->every; s >= 0 && e == cudaSuccess; --s) {
         const int64_t t0 = s * h->every;
         const int64_t len = std::min<int64_t>(h->every, h->nsteps - t0);
@@ -693,13 +916,11 @@ template <class R> cudaError_t backward_run(clb_adjoint* h, double seed, double 
             e = cudaGetLastError();
         }
         for (int64_t j = len - 1; j >= 0 && e == cudaSuccess; --j) {
-            adj_back_kernel<R><<<nb, kAdjThreads, 0, h->stream>>>(state_at<R>(h->seg, h->state_elems, j), lam, mu,
-                                                                  h->acc, k);
+            adj_back_kernel<R><<<nb, kAdjThreads, 0, h->stream>>>(state_at<R>(h->seg, h->state_elems, j), mu_next,
+                                                                  static_cast<const R*>(h->lam_final), mu, h->acc, k);
             e = cudaGetLastError();
-            if (e != cudaSuccess) break;
-            adj_transpose_kernel<R><<<nb, kAdjThreads, 0, h->stream>>>(mu, lam2, k);
-            e = cudaGetLastError();
-            std::swap(lam, lam2);
+            mu_next = mu;
+            mu = static_cast<R*>(mu == h->mu0 ? h->mu : h->mu0);
         }
     }
     double hacc[3];
@@ -733,8 +954,7 @@ clb_status clb_adjoint_destroy(clb_adjoint* h) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     h->dfree(h->ckpt);
     h->dfree(h->seg);
-    h->dfree(h->lam[0]);
-    h->dfree(h->lam[1]);
+    h->dfree(h->mu0);
     h->dfree(h->lam_final);
     h->dfree(h->mu);
     h->dfree(h->acc);
@@ -802,17 +1022,31 @@ clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, do
     }
     const size_t sb = h->state_elems * h->elem;
     h->ckpt = h->dalloc(sb * h->nckpt);
-    h->seg = h->dalloc(sb * (h->every + 1));
-    h->lam[0] = h->dalloc(sb);
-    h->lam[1] = h->dalloc(sb);
+    h->mu0 = h->dalloc(sb);
     h->lam_final = h->dalloc(sb);
     h->mu = h->dalloc(sb);
     h->nb = blocks_for((size_t)nx * ny, kAdjThreads);
-    // one block per pass when the grid fits in its shared memory, unless
-    // opts->pipeline asks for one launch per step (1)
-    h->resident = o.pipeline != 1 && res_smem(nx, ny, h->elem) <= kResSmemCap;
+    // one launch per pass, unless opts->pipeline asks for one launch per step
+    // (1), while that is faster than filling the GPU in each of two or three
+    // launches per step: see the rule's figures at kClusterNodes
+    h->resident = o.pipeline != 1 && (res_smem(nx, ny, h->elem) <= kResSmemCap ||
+                                      (h->storage == CLB_FP32_SHIFTED && (long long)nx * ny <= kClusterNodes));
+    // a pair of blocks for FP32 grids of one node per thread, with two
+    // segments in memory, or one where the allocator refuses the second
+    h->pair = h->resident && h->storage == CLB_FP32_SHIFTED && nx * ny <= kResThreads;
+    if (h->pair) {
+        const size_t one = pair_elems(nx, ny) * h->elem * h->every;
+        h->seg_bufs = h->nckpt > 1 ? 2 : 1;
+        h->seg = h->dalloc(one * h->seg_bufs);
+        if (!h->seg && h->seg_bufs == 2) {
+            h->seg_bufs = 1;
+            h->seg = h->dalloc(one);
+        }
+    } else {
+        h->seg = h->dalloc(sb * (h->every + 1));
+    }
     h->acc = static_cast<double*>(h->dalloc(std::max<size_t>(4 * (size_t)h->nb, 3 * kClusterMax) * sizeof(double)));
-    if (!h->ckpt || !h->seg || !h->lam[0] || !h->lam[1] || !h->lam_final || !h->mu || !h->acc) {
+    if (!h->ckpt || !h->seg || !h->mu0 || !h->lam_final || !h->mu || !h->acc) {
         clb_adjoint_destroy(h);
         return (clb_status)set_error(CLB_ENOMEM, "clb_adjoint_forward: device allocation failed");
     }

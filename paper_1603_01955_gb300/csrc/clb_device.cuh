@@ -339,6 +339,70 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
     }
 }
 
+// ------------------------------------------------- small periodic channels
+
+// Where node (x, y) of a periodic channel pulls its populations from, as
+// offsets into its [9][ny][nx] block, worked out once per launch: o[i] for
+// population i; at the walls f5, f6 (bottom) and f7, f8 (top) also take a
+// partner, wb / wt, with weight 1 - r.
+struct Pull {
+    int o[9];
+    int wb[2], wt[2];
+    bool bottom, top;
+};
+
+__device__ __forceinline__ Pull pull_of(int nx, int ny, int x, int y) {
+    Pull p;
+    const int nn = nx * ny;
+    const int xm = x == 0 ? nx - 1 : x - 1;
+    const int xp = x == nx - 1 ? 0 : x + 1;
+    auto at = [&](int i, int yy, int xx) { return i * nn + yy * nx + xx; };
+    p.bottom = y == 0;
+    p.top = y == ny - 1;
+    p.o[0] = at(0, y, x);
+    p.o[1] = at(1, y, xm);
+    p.o[3] = at(3, y, xp);
+    p.wb[0] = p.wb[1] = p.wt[0] = p.wt[1] = 0;
+    if (p.bottom) {
+        p.o[2] = at(4, 0, x);
+        p.o[5] = at(7, 0, x);
+        p.wb[0] = at(8, 0, xm);
+        p.o[6] = at(8, 0, x);
+        p.wb[1] = at(7, 0, xp);
+    } else {
+        p.o[2] = at(2, y - 1, x);
+        p.o[5] = at(5, y - 1, xm);
+        p.o[6] = at(6, y - 1, xp);
+    }
+    if (p.top) {
+        p.o[4] = at(2, y, x);
+        p.o[7] = at(5, y, x);
+        p.wt[0] = at(6, y, xp);
+        p.o[8] = at(6, y, x);
+        p.wt[1] = at(5, y, xm);
+    } else {
+        p.o[4] = at(4, y + 1, x);
+        p.o[7] = at(7, y + 1, xp);
+        p.o[8] = at(8, y + 1, xm);
+    }
+    return p;
+}
+
+// The pre-collision populations (Eq. 5, walls Eq. 20) through those offsets.
+template <class R>
+__device__ __forceinline__ void gather_at(const R* s, const Pull& p, R r, R rc, R (&f)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = s[p.o[i]];
+    if (p.bottom) {  // Eq. 20
+        f[5] = ln::fma(r, f[5], ln::mul(rc, s[p.wb[0]]));
+        f[6] = ln::fma(r, f[6], ln::mul(rc, s[p.wb[1]]));
+    }
+    if (p.top) {  // mirror of Eq. 20
+        f[7] = ln::fma(r, f[7], ln::mul(rc, s[p.wt[0]]));
+        f[8] = ln::fma(r, f[8], ln::mul(rc, s[p.wt[1]]));
+    }
+}
+
 // ------------------------------------------------- pressure boundary columns
 
 // A stored population field: element (i, y, x) at
