@@ -50,6 +50,7 @@ struct BatchArgs {
     const BatchChannel* ch;
     const KC<float>* kf;   // per-channel constants
     const KC<double>* kd;
+    const pr::Const* kp;   // kd in FP32 pairs
 };
 
 // A schedule's device tables: per block, the first entry and the count of its
@@ -119,6 +120,8 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchArgs a, const Sch
     const BatchChannel ch = mine ? a.ch[k] : BatchChannel{1, 1, 0};
     KC<R> c{};
     if (mine) c = kcs<R>(a)[k];
+    pr::Const kp{};
+    if (std::is_same<R, double>::value && mine) kp = a.kp[k];
     const int nx = ch.nx, ny = ch.ny, nn = nx * ny;
     const int lt = (int)threadIdx.x - sl.t0, nth = sl.threads;  // thread within the channel's range
     R* s = reinterpret_cast<R*>(smem_raw) + sl.smem_off;
@@ -178,7 +181,10 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchArgs a, const Sch
                 for (int q = 0; q < NPT; ++q) {
                     const int node = lt + q * nth;
                     if (node < nn) {
-                        collide<R, MODE_PERIODIC>(f[q], ref, c);
+                        if constexpr (std::is_same<R, double>::value)
+                            collide64<MODE_PERIODIC>(f[q], c, kp);
+                        else
+                            collide<R, MODE_PERIODIC>(f[q], ref, c);
 #pragma unroll
                         for (int i = 0; i < 9; ++i) out[i * nn + node] = f[q][i];
                     }
@@ -285,6 +291,7 @@ struct clb_batch {
     BatchChannel* dch = nullptr;
     KC<float>* dkf = nullptr;
     KC<double>* dkd = nullptr;
+    pr::Const* dkp = nullptr;
     double* dobs = nullptr;
     double g = 0, ref0 = 0, rho0 = 1, r = 0;
     int64_t step = 0;
@@ -437,7 +444,7 @@ clb_status make_sched(clb_batch* b, int npt, int packed, int block_min, BatchSch
 
 template <class T>
 cudaError_t launch_batch(clb_batch* b, const BatchSched& sc, void* state, int nsteps, cudaStream_t st) {
-    BatchArgs a{state, b->dch, b->dkf, b->dkd};
+    BatchArgs a{state, b->dch, b->dkf, b->dkd, b->dkp};
     dim3 grid(sc.nblocks), blk(sc.block);
     switch (sc.npt) {
         case 1: batch_kernel<T, 1><<<grid, blk, sc.smem, st>>>(a, sc.args, nsteps, sc.two_buffers); break;
@@ -500,6 +507,7 @@ clb_status clb_batch_destroy(clb_batch* b) {
     b->dfree(b->dch);
     b->dfree(b->dkf);
     b->dfree(b->dkd);
+    b->dfree(b->dkp);
     b->dfree(b->dobs);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
@@ -556,6 +564,7 @@ clb_status clb_batch_create(int n, const int* nx, const int* ny, const double* k
     long long off = 0;
     std::vector<KC<float>> kf(n);
     std::vector<KC<double>> kd(n);
+    std::vector<pr::Const> kp(n);
     for (int k = 0; k < n; ++k) {
         b->nx.push_back(nx[k]);
         b->ny.push_back(ny[k]);
@@ -575,6 +584,7 @@ clb_status clb_batch_create(int n, const int* nx, const int* ny, const double* k
         derive_constants(sa);
         kf[k] = sa.kf;
         kd[k] = sa.kd;
+        kp[k] = sa.kp;
     }
     b->total = off;
     if (o.stream) {
@@ -590,14 +600,16 @@ clb_status clb_batch_create(int n, const int* nx, const int* ny, const double* k
     b->dch = static_cast<BatchChannel*>(b->dalloc(n * sizeof(BatchChannel)));
     b->dkf = static_cast<KC<float>*>(b->dalloc(n * sizeof(KC<float>)));
     b->dkd = static_cast<KC<double>*>(b->dalloc(n * sizeof(KC<double>)));
+    b->dkp = static_cast<pr::Const*>(b->dalloc(n * sizeof(pr::Const)));
     b->dobs = static_cast<double*>(b->dalloc(9 * (size_t)n * sizeof(double)));
-    if (!b->state || !b->dch || !b->dkf || !b->dkd || !b->dobs) {
+    if (!b->state || !b->dch || !b->dkf || !b->dkd || !b->dkp || !b->dobs) {
         clb_batch_destroy(b);
         return (clb_status)set_error(CLB_ENOMEM, "clb_batch_create: device allocation failed");
     }
     cudaError_t e = cudaMemcpyAsync(b->dch, b->hch.data(), n * sizeof(BatchChannel), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dkf, kf.data(), n * sizeof(KC<float>), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dkd, kd.data(), n * sizeof(KC<double>), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dkp, kp.data(), n * sizeof(pr::Const), cudaMemcpyHostToDevice, b->stream);
     // initial state f^eq(rho_out, 0) = w_i rho_out: zero deviations (FP32) or w_i rho_out (FP64)
     if (e == cudaSuccess) e = cudaMemsetAsync(b->state, 0, b->total * elem, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -750,7 +762,7 @@ clb_status clb_batch_step(clb_batch* b, int64_t n) {
 
 clb_status clb_batch_observables(clb_batch* b, clb_scalars* s) {
     if (!b || !s) return (clb_status)set_error(CLB_EINVAL, "clb_batch_observables: NULL argument");
-    BatchArgs a{b->state, b->dch, b->dkf, b->dkd};
+    BatchArgs a{b->state, b->dch, b->dkf, b->dkd, b->dkp};
     if (b->storage == CLB_FP64)
         batch_obs_kernel<double><<<b->n, kObsThreads, 0, b->stream>>>(a, b->ref0, b->g, b->dobs);
     else

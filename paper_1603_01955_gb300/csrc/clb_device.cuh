@@ -339,6 +339,39 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
     }
 }
 
+// The FP64 collision of a node (densities, R = 0): in FP32 pairs where the
+// node is near enough to equilibrium (pair.cuh), else in plain FP64, out of
+// line: few nodes take it, and its registers are not the fast path's.
+template <int MODE>
+__device__ __noinline__ void collide_plain64(double* f, const KC<double>* c, const double* rho_kn) {
+    double d[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) d[i] = f[i];
+    collide<double, MODE>(d, 0.0, *c, rho_kn);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = d[i];
+}
+template <int MODE>
+__device__ __forceinline__ void collide64(double (&f)[9], const KC<double>& c, const pr::Const& kp,
+                                          const double* rho_kn = nullptr) {
+    float R;
+    pr::P d[9], o[9];
+    if (pr::deviations(f, R, d)) {
+        pr::P kn{0.0f, 0.0f};
+        if (MODE == MODE_PRESSURE && rho_kn) kn = pr::split(*rho_kn);
+        pr::collide<MODE == MODE_PERIODIC>(R, d, kp, MODE == MODE_PRESSURE && rho_kn ? &kn : nullptr, o);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = pr::dadd(f[i], pr::join(pr::norm(o[i])));
+    } else {
+        double t[9], kn = rho_kn ? *rho_kn : 0.0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) t[i] = f[i];
+        collide_plain64<MODE>(t, &c, rho_kn ? &kn : nullptr);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = t[i];
+    }
+}
+
 // ------------------------------------------------- small periodic channels
 
 // Where node (x, y) of a periodic channel pulls its populations from, as
@@ -418,27 +451,30 @@ template <class T> struct Field {
 // end columns.
 template <class R, class At>
 __device__ __forceinline__ void gather_node_at(const KC<R>& c, int rt, At at, R (&o)[9]) {
-    const R sha = c.sha, shd = c.shd;  // source at x-1; the source at x+1 gets the negative
+    // source at x-1; the source at x+1 gets the negative (FP64: R = 0, none)
+    auto left = [&](R v, R s) { return std::is_same<R, double>::value ? v : v + s; };
+    auto right = [&](R v, R s) { return std::is_same<R, double>::value ? v : v - s; };
+    const R sha = c.sha, shd = c.shd;
     o[0] = at(0, 0, 0);
-    o[1] = at(1, 0, -1) + sha;
-    o[3] = at(3, 0, 1) - sha;
+    o[1] = left(at(1, 0, -1), sha);
+    o[3] = right(at(3, 0, 1), sha);
     if (rt & ROW_BOTTOM) {
         o[2] = at(4, 0, 0);
-        o[5] = c.r * at(7, 0, 0) + c.rc * (at(8, 0, -1) + shd);
-        o[6] = c.r * at(8, 0, 0) + c.rc * (at(7, 0, 1) - shd);
+        o[5] = c.r * at(7, 0, 0) + c.rc * left(at(8, 0, -1), shd);
+        o[6] = c.r * at(8, 0, 0) + c.rc * right(at(7, 0, 1), shd);
     } else {
         o[2] = at(2, -1, 0);
-        o[5] = at(5, -1, -1) + shd;
-        o[6] = at(6, -1, 1) - shd;
+        o[5] = left(at(5, -1, -1), shd);
+        o[6] = right(at(6, -1, 1), shd);
     }
     if (rt & ROW_TOP) {
         o[4] = at(2, 0, 0);
-        o[7] = c.r * at(5, 0, 0) + c.rc * (at(6, 0, 1) - shd);
-        o[8] = c.r * at(6, 0, 0) + c.rc * (at(5, 0, -1) + shd);
+        o[7] = c.r * at(5, 0, 0) + c.rc * right(at(6, 0, 1), shd);
+        o[8] = c.r * at(6, 0, 0) + c.rc * left(at(5, 0, -1), shd);
     } else {
         o[4] = at(4, 1, 0);
-        o[7] = at(7, 1, 1) - shd;
-        o[8] = at(8, 1, -1) + shd;
+        o[7] = right(at(7, 1, 1), shd);
+        o[8] = left(at(8, 1, -1), shd);
     }
 }
 
@@ -483,6 +519,67 @@ __device__ __forceinline__ void rebuild_nodes(const KC<R>& c, int x, bool inlet,
     for (int i = 0; i < 9; ++i) out[i] = eb[i] + (n1[i] - e1[i]);
 }
 
+// The same of an FP64 channel, in FP32 pairs where both neighbours are near
+// enough to equilibrium (pair.cuh).  Its two halves: a neighbour's density and
+// velocity, and the populations of the end column from the first neighbour's.
+struct Macro64 {
+    float R;
+    pr::P rho, drho, ux, uy;
+};
+__device__ __forceinline__ bool macro64(const double (&n)[9], Macro64& v) {
+    pr::P d[9];
+    pr::Moments m;
+    const bool fine = pr::deviations(n, v.R, d);
+    pr::moments(v.R, d, m);
+    pr::velocity(m, v.ux, v.uy);
+    v.rho = m.rho;
+    v.drho = m.drho;
+    return fine;
+}
+__device__ __forceinline__ void end_column64(const double (&n1)[9], const Macro64& m1, pr::P u2x, pr::P u2y, double rho_b,
+                                             double* out) {
+    pr::P o[9];
+    const pr::P dr = pr::norm(pr::sub(pr::split(rho_b - (double)m1.R), m1.drho));
+    const pr::P vx = pr::norm(pr::sub(pr::twice(m1.ux), u2x)), vy = pr::norm(pr::sub(pr::twice(m1.uy), u2y));
+    pr::eq_difference(m1.rho, dr, m1.ux, m1.uy, vx, vy, o);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) out[i] = pr::dadd(n1[i], pr::join(pr::norm(o[i])));
+}
+// Whether the end column's own density is near enough to its neighbour's.
+__device__ __forceinline__ bool end_fine64(const Macro64& m1, double rho_b) {
+    const float d = fabsf((float)rho_b - m1.R);
+    return d <= m1.R * (1.0f / 64.0f);
+}
+static __device__ __noinline__ void rebuild_plain64(const KC<double>* c, int x, bool inlet, const double* a, const double* b,
+                                             double* out) {
+    double n1[9], n2[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        n1[i] = a[i];
+        n2[i] = b[i];
+    }
+    rebuild_nodes<double>(*c, x, inlet, n1, n2, out);
+}
+__device__ __forceinline__ void rebuild_nodes64(const KC<double>& c, int x, bool inlet, const double (&n1)[9],
+                                                const double (&n2)[9], double* out) {
+    Macro64 m1, m2;
+    const bool f1 = macro64(n1, m1), f2 = macro64(n2, m2);
+    const double rho_b = inlet ? c.drho_in : c.drho_out;
+    if (f1 && f2 && end_fine64(m1, rho_b)) {
+        end_column64(n1, m1, m2.ux, m2.uy, rho_b, out);
+    } else {
+        double a[9], b[9], t[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            a[i] = n1[i];
+            b[i] = n2[i];
+        }
+        rebuild_plain64(&c, x, inlet, a, b, t);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) out[i] = t[i];
+    }
+}
+
 // The same from the populations in global memory.
 template <class T, class R>
 __device__ __forceinline__ void rebuild_column(const SweepArgs& a, const KC<R>& c, const Field<T> f, int x, int y,
@@ -491,7 +588,10 @@ __device__ __forceinline__ void rebuild_column(const SweepArgs& a, const KC<R>& 
     R n1[9], n2[9];
     gather_node<T, R>(a, c, f, x + dir, y, n1);
     gather_node<T, R>(a, c, f, x + 2 * dir, y, n2);
-    rebuild_nodes<R>(c, x, inlet, n1, n2, out);
+    if constexpr (std::is_same<R, double>::value)
+        rebuild_nodes64(c, x, inlet, n1, n2, out);
+    else
+        rebuild_nodes<R>(c, x, inlet, n1, n2, out);
 }
 
 }  // namespace clb

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include "pair.cuh"
+
 namespace clb {
 
 enum : int { MODE_PERIODIC = 0, MODE_PRESSURE = 1 };
@@ -75,9 +77,10 @@ struct SweepArgs {
     // them; the collision is homogeneous in the densities, so the results are
     // the scaled results bit for bit.
     KC<float> ks;
+    pr::Const kp;  // kd in FP32 pairs, for the FP64 collision
 };
 
-// Fill a.kf, a.kd and a.ks from the double fields of a.
+// Fill a.kf, a.kd, a.ks and a.kp from the double fields of a.
 void derive_constants(SweepArgs& a);
 
 // s_v (Eq. 18) and s_q (Eq. 21) at a Knudsen number, N = ny.

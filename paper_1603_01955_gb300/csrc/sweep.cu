@@ -33,14 +33,14 @@
 // compiler for the FP32/16-bit sweeps, which caps their registers: 4 -> 64
 // registers, 8 blocks of 128 threads per SM.  These kernels are bound by DRAM
 // latency, and the occupancy this buys outweighs a 36-byte spill.
-// CLB_SWEEP_MIN_BLOCKS_FP64: the same for the FP64 sweep (FP64-pipe bound).
+// CLB_SWEEP_MIN_BLOCKS_FP64: the same for the FP64 sweep (see pair.cuh).
 // CLB_SWEEP_STREAMING: 1 = evict-first (.cs) hints on the population loads
 // and stores, which are touched exactly once per step (measured slower).
 #ifndef CLB_SWEEP_MIN_BLOCKS
 #define CLB_SWEEP_MIN_BLOCKS 4
 #endif
 #ifndef CLB_SWEEP_MIN_BLOCKS_FP64
-#define CLB_SWEEP_MIN_BLOCKS_FP64 2
+#define CLB_SWEEP_MIN_BLOCKS_FP64 4
 #endif
 #ifndef CLB_SWEEP_STREAMING
 #define CLB_SWEEP_STREAMING 0
@@ -288,7 +288,10 @@ __global__ void __launch_bounds__(256, MinBlocks<T>::value) sweep_kernel(const S
             R* out = static_cast<R*>(a.rc_out) + (y == a.yc0 ? 0 : a.rc_stride);
             out[x0 + k] = ref + dr;
         }
-        collide<R, MODE>(d, ref, c, centre_kn ? &rk[k] : nullptr);
+        if constexpr (std::is_same<T, double>::value)
+            collide64<MODE>(d, c, a.kp, centre_kn ? &rk[k] : nullptr);
+        else
+            collide<R, MODE>(d, ref, c, centre_kn ? &rk[k] : nullptr);
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i][k] = d[i];
     }
@@ -369,6 +372,10 @@ template <typename R> static void fill(KC<R>& c, const SweepArgs& a) {
 void derive_constants(SweepArgs& a) {
     fill(a.kf, a);
     fill(a.kd, a);
+    const KC<double>& d = a.kd;
+    a.kp = pr::Const{pr::pair_of(d.s3_12), pr::pair_of(d.s8_4), pr::pair_of(d.sv_4), pr::pair_of(d.sq_4),
+                     pr::pair_of(d.A),     pr::pair_of(d.B),    pr::pair_of(d.A316), pr::pair_of(d.CA),
+                     pr::pair_of(d.fx),    pr::pair_of(d.hfx)};
     // densities scale, 1/densities scale inversely, rates and velocities do not
     KC<float>& k = a.ks;
     k = a.kf;

@@ -210,7 +210,10 @@ __global__ void __launch_bounds__(kTileThreads + kEndThreads, 1)
             f[8] = ln::fma(c.r, f[8], ln::mul(c.rc, s5));
         }
     };
-    auto ref_of = [&](int x) { return MODE == MODE_PRESSURE ? ln::fma(c.slope, R(lo + x), c.ref0) : c.ref0; };
+    auto ref_of = [&](int x) {
+        if (std::is_same<T, double>::value) return R(0);
+        return MODE == MODE_PRESSURE ? ln::fma(c.slope, R(lo + x), c.ref0) : c.ref0;
+    };
     // the density that sets the column's Knudsen number, and this step's own
     // at the centre rows
     auto centre_in = [&](int x, int par) {
@@ -236,20 +239,25 @@ __global__ void __launch_bounds__(kTileThreads + kEndThreads, 1)
             rk = centre_in(x, par);
             centre_out(x, row, par, ref, f);
         }
-        collide<R, MODE>(f, ref, c, centre_kn ? &rk : nullptr);
+        if constexpr (std::is_same<T, double>::value)
+            collide64<MODE>(f, c, a.kp, centre_kn ? &rk : nullptr);
+        else
+            collide<R, MODE>(f, ref, c, centre_kn ? &rk : nullptr);
         put(x, row, f);
     };
     constexpr bool kEnds = MODE == MODE_PRESSURE;
     // Item e of the end columns: two lanes per node.  Lane 0 gathers the first
     // interior neighbour and keeps its non-equilibrium part, lane 1 the second,
     // for the velocity, and then the imposed equilibrium (rebuild_nodes, with
-    // its two halves side by side).  True in lane 0 of a node of this tile.
+    // its two halves side by side).  Whole warps call it; true in lane 0 of a node
+    // of this tile.
     auto rebuild_end = [&](int e, int& xe, int& row, R (&f)[9]) {
+        constexpr unsigned kAll = 0xffffffffu;
+        __syncwarp();
         const int half = e & 1, q = e >> 1;
         const bool right = q >= ny;
-        row = right ? q - ny : q;
-        const unsigned lanes = __activemask();
-        const bool on = right ? fixr : fixl;
+        const bool on = e < 4 * ny && (right ? fixr : fixl);
+        row = !on ? 0 : right ? q - ny : q;
         const int dir = right ? -1 : 1;
         xe = right ? cols - 1 : 0;
         const int xs = on ? xe + (half ? 2 : 1) * dir : min(1, cols - 1);
@@ -260,30 +268,58 @@ __global__ void __launch_bounds__(kTileThreads + kEndThreads, 1)
         else
 #pragma unroll
             for (int i = 0; i < 9; ++i) v[i] = R(1);
-        R dr, jx, jy;
-        macro_dev(v, dr, jx, jy);
-        const R rho = c.ref0 + c.slope * R(lo + xs) + dr;
-        const R ux = jx / rho, uy = jy / rho;
-        const R vx = __shfl_xor_sync(lanes, ux, 1), vy = __shfl_xor_sync(lanes, uy, 1);
-        const R drb = right ? c.drho_out : c.drho_in;
-        const R rb = c.ref0 + c.slope * R(lo + xe) + drb;
-        R eq[9];
-        feq_dev(half ? drb : dr, half ? rb : rho, half ? R(2) * vx - ux : ux, half ? R(2) * vy - uy : uy, eq);
+        if constexpr (std::is_same<T, double>::value) {
+            Macro64 mac;
+            const bool fine = macro64(v, mac);
+            const double rho_b = right ? c.drho_out : c.drho_in;
+            // (every lane takes part in every shuffle: none behind a condition)
+            const int fine2 = __shfl_xor_sync(kAll, (int)fine, 1);
+            const bool both = fine && fine2 && end_fine64(mac, rho_b);  // of lane 0
+            const pr::P u2x{__shfl_xor_sync(kAll, mac.ux.h, 1), __shfl_xor_sync(kAll, mac.ux.l, 1)};
+            const pr::P u2y{__shfl_xor_sync(kAll, mac.uy.h, 1), __shfl_xor_sync(kAll, mac.uy.l, 1)};
+            double n2[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const R eb = __shfl_xor_sync(lanes, eq[i], 1);
-            f[i] = eb + (v[i] - eq[i]);
+            for (int i = 0; i < 9; ++i) n2[i] = __shfl_xor_sync(kAll, v[i], 1);
+            if (on && !half) {
+                if (both) {
+                    end_column64(v, mac, u2x, u2y, rho_b, f);
+                } else {
+                    double n1[9], t[9];
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) n1[i] = v[i];
+                    rebuild_plain64(&c, lo + xe, !right, n1, n2, t);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) f[i] = t[i];
+                }
+            }
+            return on && !half;
+        } else {
+            R dr, jx, jy;
+            macro_dev(v, dr, jx, jy);
+            const R rho = c.ref0 + c.slope * R(lo + xs) + dr;
+            const R ux = jx / rho, uy = jy / rho;
+            const R vx = __shfl_xor_sync(kAll, ux, 1), vy = __shfl_xor_sync(kAll, uy, 1);
+            const R drb = right ? c.drho_out : c.drho_in;
+            const R rb = c.ref0 + c.slope * R(lo + xe) + drb;
+            R eq[9];
+            feq_dev(half ? drb : dr, half ? rb : rho, half ? R(2) * vx - ux : ux, half ? R(2) * vy - uy : uy, eq);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const R eb = __shfl_xor_sync(kAll, eq[i], 1);
+                f[i] = eb + (v[i] - eq[i]);
+            }
+            return on && !half;
         }
-        return on && !half;
     };
 
+    const int end_items = (4 * ny + 31) / 32 * 32;  // whole warps
     for (int t = 0; t < nsteps; ++t) {
         // columns whose neighbours are still exact after t steps
         const int al = fixl ? (kEnds ? 1 : 0) : t + 1, ar = fixr ? cols - (kEnds ? 1 : 0) : cols - t - 1;
         const int par = t & 1;
         if constexpr (PACK) {
             if (kEnds && end_thread && (fixl || fixr))
-                for (int e = threadIdx.x - p.main; e < 4 * ny; e += blockDim.x - p.main) {
+                for (int e = threadIdx.x - p.main; e < end_items; e += blockDim.x - p.main) {
                     int x, row;
                     R f[9];
                     if (rebuild_end(e, x, row, f)) finish(x, row, par, f);
@@ -321,7 +357,7 @@ __global__ void __launch_bounds__(kTileThreads + kEndThreads, 1)
             // one loop and one copy of the collision's code for both kinds of thread
             const bool ends = kEnds && end_thread;
             const int step = ends ? blockDim.x - p.main : p.cpp;
-            const int until = ends ? (fixl || fixr ? 4 * ny : 0) : mine ? ar : 0;
+            const int until = ends ? (fixl || fixr ? end_items : 0) : mine ? ar : 0;
             for (int k = ends ? threadIdx.x - p.main : x0; k < until; k += step) {
                 int x = k, row = y;
                 R f[9];
@@ -407,22 +443,26 @@ template <class F> cudaError_t with_tile(int storage, int mode, const TilePlan& 
 // 1601 x 16 pressure FP32: w 11, h 9, expected 1.4, measured 1.25 us per step,
 // against 2.9 us; 801 x 8 periodic 0.68 against 2.6; 4 x 32 in one block 0.33
 // against 2.8; 6401 x 64 stays with the direct sweep (7.2 against 6.3 us).
-// FP64 is bound by the FP64 pipe (64 cycles per warp and instruction), not by
-// latency: only a channel of one warp per scheduler gains (7.0 against 8.3 us
-// for 4 x 32), and halo columns cost more than launches.
+// FP64 (pair.cuh), in the same way: a step costs 1.2 us, 3.2 us with the end of
+// a pressure channel, and 10 ns per node; the direct sweep 4.6 or 8.2 us and
+// 0.048 ns per node.  801 x 8 pressure: 5.3 us per step, against 8.1; periodic
+// 2.8 against 4.6; 4 x 32 in one block 2.0 against 4.7; 2101 x 33 stays with the
+// direct sweep (9.0 against 7.7).
 TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_cap) {
     TilePlan best;
     if (ny > kTileThreads || sms < 1) return best;
     const size_t elem = storage == 0 ? 8 : storage == 1 ? 4 : 2, relem = storage == 0 ? 8 : 4;
     const int cs = ny | 1;
-    double best_t = 0.9 * (2500.0 + 0.01 * nx * ny);
+    const bool f64 = storage == 0, press = mode == MODE_PRESSURE;
+    double best_t = 0.9 * (f64 ? (press ? 8200.0 : 4600.0) + 0.048 * nx * ny : 2500.0 + 0.01 * nx * ny);
     auto consider = [&](int blocks, int h, bool whole) {
         const int w = (nx + blocks - 1) / blocks, cols = whole ? nx : w + 2 * h;
         const bool big = (size_t)cols * cs > plane_of(elem, false);
         const size_t smem = tile_smem(big, cols, elem, relem);
         if (smem > smem_cap || (size_t)cols * cs > plane_of(elem, big)) return;
-        double step = 200.0 + 1.5 * ny * (whole ? nx : w + h);
-        if (mode == MODE_PRESSURE) step = std::max(step, 1050.0);
+        const double nodes = (double)ny * (whole ? nx : w + h);
+        double step = f64 ? (press ? 3200.0 : 1200.0) + 10.0 * nodes : 200.0 + 1.5 * nodes;
+        if (press && !f64) step = std::max(step, 1050.0);
         const double ns = step + (whole ? 0.0 : (2500.0 + 0.04 * 9 * elem * ny * (cols + w)) / h);
         if (ns >= best_t) return;
         best_t = ns;
@@ -434,19 +474,15 @@ TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_
         // one column per thread and pass, or a pair in packed FP32 where the
         // columns are more than one pass
         const int fit = kTileThreads / ny;  // columns (or pairs) that the threads cover
-        t.pack = storage != 0 && cols > fit;
+        t.pack = !f64 && cols > fit;
         const int units = t.pack ? (cols + 1) / 2 : cols, passes = (units + fit - 1) / fit;
         t.cpp = (units + passes - 1) / passes;
         t.main = (t.cpp * ny + 31) / 32 * 32;
-        t.threads = t.main + (mode == MODE_PRESSURE ? std::min(kEndThreads, (4 * ny + 31) / 32 * 32) : 0);
+        t.threads = t.main + (press ? std::min(kEndThreads, (4 * ny + 31) / 32 * 32) : 0);
         t.blocks = blocks;
         t.smem = smem;
         best = t;
     };
-    if (storage == 0) {
-        if (nx * ny <= 128 && mode == MODE_PERIODIC) consider(1, kTileMaxSteps, true);
-        return best;
-    }
     consider(1, kTileMaxSteps, true);
     // a block that holds an end of a pressure channel needs the three columns
     // beside it to stay exact (the end is rebuilt from columns 1 and 2, which
