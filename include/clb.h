@@ -97,7 +97,11 @@ typedef struct {
      * copies, tile shape 0..2 of the table in sweep_tma.cu (2: 512 consumer
      * threads x 2 nodes, 3 stages; 3: 128 x 4 nodes, 2 stages; 4: 256 x 4
      * nodes, 3 stages), tiles claimed dynamically by the blocks of a
-     * persistent grid.  All give bit-identical results. */
+     * persistent grid.  With all of pipeline, vec and block_x 0, small
+     * channels advance several steps per launch in shared memory and FP32
+     * pressure channels of 500,000 nodes and at least 2000 columns two steps
+     * per launch; the engine named above then takes what is left over.  All
+     * give bit-identical results. */
     int pipeline;
     /* Local Knudsen number of a pressure channel (Sec. 3.2): 0 = from the
      * node's own pressure (default), 1 = from the centreline pressure p(x) of

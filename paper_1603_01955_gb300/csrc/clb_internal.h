@@ -117,6 +117,11 @@ cudaError_t launch_sweep_tma(int storage, int mode, int variant, const SweepArgs
                              unsigned* sched, unsigned* status);
 int tma_variant_count();
 
+// Two steps per launch of a large FP32 pressure channel (march.cu), and its
+// opt-in to shared memory on the current device.
+cudaError_t march_opt_in();
+cudaError_t launch_march(int sms, const SweepArgs& a, cudaStream_t st);
+
 // Several steps per launch of a small channel held in shared memory (tile.cu).
 struct TilePlan {
     int h = 0;            // steps per launch at most (0: no plan)

@@ -86,6 +86,7 @@ struct clb_sim {
     int withhold_tile = -1; // testing: TMA tile withheld in the first launch
     int graph_steps = 0;    // sweeps per replayed CUDA graph (0: no replay); even
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // per parity of `cur` at the chunk start
+    int march_sms = 0;      // SMs, if two steps per launch (march.cu): larger channels, default engine
     TilePlan tile;          // several steps per launch (tile.h > 0): small channels, default engine
     int kn_mode = 0;        // 1: centreline Knudsen number (pressure channel)
     void* rc = nullptr;     // centreline densities: [2 sides][2 rows][rc_stride], compute type
@@ -706,12 +707,26 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
         s->pipeline = 1;  // small channels: the direct sweep has the shorter latency per step
     else
         s->pipeline = (o.storage == CLB_FP32_SHIFTED) ? 2 : 3;
-    // small channels of the default engine: several steps per launch
-    if (o.pipeline == 0 && o.vec == 0 && o.block_x == 0 && s->pipeline == 1 && o.test_withhold_tile < 0) {
+    // the default engine takes several steps per launch where that is faster:
+    // - FP32 pressure channels of half a million nodes and more, two (march.cu;
+    //   us per step, against one per launch: 25601 x 256 47.8 / 72.5; 4097 x 256
+    //   10.0 / 18.5; 8001 x 80 7.1 / 8.5; 7001 x 70 6.6 / 6.8; 6401 x 64 6.1 /
+    //   6.2), unless they are narrow (2000 x 400 9.7 / 10.4; 1000 x 800 12.2 /
+    //   10.7: one strip in eight holds an end column, which is slower);
+    // - small channels, more (tile.cu).
+    const bool stock = o.pipeline == 0 && o.vec == 0 && o.block_x == 0 && o.test_withhold_tile < 0;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (stock && o.storage == CLB_FP32_SHIFTED && drive == CLB_DRIVE_PRESSURE && s->kn_mode == 0 && nx >= 2000 &&
+        (long long)nx * ny >= 500000) {
+        if (march_opt_in() == cudaSuccess)
+            s->march_sms = std::max(sms, 1);
+        else
+            cudaGetLastError();
+    } else if (stock && s->pipeline == 1) {
         const int mode = drive == CLB_DRIVE_PRESSURE ? MODE_PRESSURE : MODE_PERIODIC;
-        int dev = 0, sms = 0, cap = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int cap = 0;
         cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         s->tile = plan_tiles(o.storage, mode, nx, ny, sms, (size_t)std::max(cap, 0));
         if (s->tile.h > 0 && tile_opt_in(o.storage, mode, s->tile) != cudaSuccess) {
@@ -835,6 +850,7 @@ static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur, in
     a.rc_in = static_cast<const char*>(s->rc) + cur * rc_side;
     a.rc_out = static_cast<char*>(s->rc) + (cur ^ 1) * rc_side;
     a.tile_order = cur;  // alternate the TMA sweep's tile order with the buffers
+    if (steps == 2 && s->march_sms) return launch_march(s->march_sms, a, s->stream);
     if (s->tile.h > 0) return launch_tiles(s->storage, mode, s->tile, a, steps, s->stream);
     return s->pipeline >= 2 ? launch_sweep_tma(s->storage, mode, s->pipeline - 2, a, s->stream, s->sched, s->status)
                             : launch_sweep(s->storage, mode, s->vec, s->block_x, a, s->stream);
@@ -844,7 +860,7 @@ static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur, in
 // most the steps the engine takes at once; `even`: an even number of launches,
 // so that they end on the buffer they started from.  *done counts the steps queued.
 static cudaError_t launch_steps(clb_sim* s, SweepArgs& a, int mode, int* cur, int64_t n, bool even, int64_t* done) {
-    const int64_t most = s->tile.h > 0 ? s->tile.h : 1;
+    const int64_t most = s->tile.h > 0 ? s->tile.h : s->march_sms ? 2 : 1;
     int64_t launches = (n + most - 1) / most;
     if (even && launches % 2) ++launches;
     *done = 0;
