@@ -314,28 +314,30 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
     d[6] = add(d[6], sub(e6, gm));
     d[8] = add(d[8], add(e6, gm));
     if (MODE == MODE_PERIODIC) {
-        // source S = T^-1 S^ (Eq. 9-10), T^-1 in closed form as tinv_apply
-        const L fx = bc<L>(c.fx), two = k(2.0), qt = k(0.25);
+        // source S = T^-1 S^ (Eq. 9-10), T^-1 in closed form as tinv_apply; the
+        // powers of two are taken together at the end, in the fused
+        // multiply-adds (m3, m8 and the differences at half their size)
+        const L fx = bc<L>(c.fx), half = k(0.5), qt = k(0.25);
         const L m1 = prod(rho, fx);
-        const L m3 = mul(two, prod(rho, mul(ux, fx)));  // = m4
+        const L m3 = prod(rho, mul(ux, fx));  // half of m3 = m4
         const L m5 = prod(rho, mul(uy, fx));
-        const L m6 = prod(rho, mul(mul(two, fx), uxy));
+        const L m6 = prod(rho, mul(mul(k(2.0), fx), uxy));
         const L m7 = prod(rho, mul(fx, uy2));
-        const L m8 = mul(two, prod(rho, mul(uxy, mul(fx, uy))));
+        const L m8 = prod(rho, mul(uxy, mul(fx, uy)));  // half of m8
         const L cm = fma(k(-2.0), m8, m3);
         const L b4 = add(cm, m3), e4 = sub(cm, m3);
-        const L a17 = mul(two, sub(m1, m7)), a26 = mul(k(-2.0), m6);
+        const L a17 = sub(m1, m7);
         const L p56 = add(m5, m6), n56 = sub(m6, m5);
-        const L p78 = add(m7, m8), n78 = sub(m8, m7);
-        d[0] = add(d[0], sub(m8, m3));  // S_0 = m0 - m3 + m8 with m0 = 0
-        d[1] = add(d[1], mul(qt, add(b4, a17)));
-        d[3] = add(d[3], mul(qt, sub(b4, a17)));
-        d[2] = add(d[2], mul(qt, add(e4, a26)));
-        d[4] = add(d[4], mul(qt, sub(e4, a26)));
-        d[5] = add(d[5], mul(qt, add(p56, p78)));
-        d[6] = add(d[6], mul(qt, add(n56, n78)));
-        d[7] = add(d[7], mul(qt, sub(n78, n56)));
-        d[8] = add(d[8], mul(qt, sub(p78, p56)));
+        const L p78 = fma(k(2.0), m8, m7), n78 = fma(k(2.0), m8, neg(m7));
+        d[0] = fma(k(2.0), sub(m8, m3), d[0]);  // S_0 = m0 - m3 + m8 with m0 = 0
+        d[1] = fma(half, add(b4, a17), d[1]);
+        d[3] = fma(half, sub(b4, a17), d[3]);
+        d[2] = fma(half, sub(e4, m6), d[2]);
+        d[4] = fma(half, add(e4, m6), d[4]);
+        d[5] = fma(qt, add(p56, p78), d[5]);
+        d[6] = fma(qt, add(n56, n78), d[6]);
+        d[7] = fma(qt, sub(n78, n56), d[7]);
+        d[8] = fma(qt, sub(p78, p56), d[8]);
     }
 }
 
