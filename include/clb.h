@@ -329,9 +329,9 @@ typedef struct clb_adjoint clb_adjoint; /* opaque */
  * sums are FP64, or FP32 pairs of 48 bits).  r < 0 takes r_b from Eq. 21 with
  * opts->sigma (the gradient is still with respect to r_b).  Device memory:
  * (ceil(nsteps/C) + C + 4) states of 9 nx ny elements; for FP32 grids of at most
- * 512 nodes (ceil(nsteps/C) + 2 C + 3) states and 16 C nx elements, or with C
- * in the place of 2 C where the allocator refuses that.  Synchronises.
- * nx * ny <= 2^22.
+ * 512 nodes (ceil(nsteps/C) + 2 C + 3) states and 16 C nx elements, or half of
+ * 2 C and 16 C where the allocator refuses that, or the former where it refuses
+ * that too.  Synchronises.  nx * ny <= 2^22.
  * Engine: a grid whose two states fit in one block's shared memory
  * (2 * 9 nx ny elements <= about 200 KB: 2800 nodes in FP32) runs the
  * forward pass as one launch of one block and each backward pass as one

@@ -1032,7 +1032,8 @@ clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, do
     h->resident = o.pipeline != 1 && (res_smem(nx, ny, h->elem) <= kResSmemCap ||
                                       (h->storage == CLB_FP32_SHIFTED && (long long)nx * ny <= kClusterNodes));
     // a pair of blocks for FP32 grids of one node per thread, with two
-    // segments in memory, or one where the allocator refuses the second
+    // segments in memory, or one where the allocator refuses the second; a
+    // cluster, whose segment is plain states, where it refuses that too
     h->pair = h->resident && h->storage == CLB_FP32_SHIFTED && nx * ny <= kResThreads;
     if (h->pair) {
         const size_t one = pair_elems(nx, ny) * h->elem * h->every;
@@ -1042,9 +1043,9 @@ clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, do
             h->seg_bufs = 1;
             h->seg = h->dalloc(one);
         }
-    } else {
-        h->seg = h->dalloc(sb * (h->every + 1));
+        h->pair = h->seg != nullptr;
     }
+    if (!h->seg) h->seg = h->dalloc(sb * (h->every + 1));
     h->acc = static_cast<double*>(h->dalloc(std::max<size_t>(4 * (size_t)h->nb, 3 * kClusterMax) * sizeof(double)));
     if (!h->ckpt || !h->seg || !h->mu0 || !h->lam_final || !h->mu || !h->acc) {
         clb_adjoint_destroy(h);

@@ -70,3 +70,36 @@ def test_second_segment_refused(clb):
     J1, g1, refused = run(2 * one_segment - 1)
     assert refused == 1
     assert (J1, g1) == (J, g)
+
+
+def test_wall_terms_refused(clb):
+    """A segment of pulled populations and wall terms is larger than its plain
+    states where the grid is wide: the cluster, which keeps the states, takes
+    the backward pass where the allocator refuses the former."""
+    import torch
+
+    def run(limit):
+        refused = []
+
+        def alloc(n, ctx):
+            if n > limit:
+                refused.append(n)
+                return None
+            return torch.cuda.caching_allocator_alloc(int(n))
+
+        def free(p, ctx):
+            torch.cuda.caching_allocator_delete(int(p))
+
+        o = clb.clb_opts_default()
+        hooks = (clb.ALLOC_FN(alloc), clb.FREE_FN(free))
+        o.alloc, o.free = hooks
+        h, J = clb.clb_adjoint_forward(16, 4, 0.3, 2.0, 0.8, 2e-5, 500, 50, o)
+        g = clb.clb_adjoint_backward(h)
+        clb.clb_adjoint_destroy(h)
+        return (J, *g), len(refused)
+
+    want, refused = run(1 << 40)
+    assert refused == 0
+    got, refused = run(4 * 51 * 9 * 64)
+    assert refused == 2
+    assert got == pytest.approx(want, rel=1e-5)
