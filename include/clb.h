@@ -115,8 +115,9 @@ typedef struct {
     /* CUDA-graph replay of clb_step for channels whose sweeps are short
      * enough for launch overhead to matter: chunks of this many consecutive
      * sweeps are captured once (per buffer parity) and replayed.  0 =
-     * default (64 for channels below 2^20 nodes, off above; off with the
-     * testing option), < 0 = off, > 0 = chunk length.
+     * default (64 steps for channels below 2^20 nodes, or the next even
+     * number of whole launches where a launch takes several; off above, and
+     * with the testing option), < 0 = off, > 0 = chunk length.
      * Results are identical with or without replay. */
     int graph_steps;
 } clb_opts;

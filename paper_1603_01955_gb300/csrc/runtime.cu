@@ -741,8 +741,10 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
             k = o.graph_steps;
         else if (o.graph_steps == 0)
             k = ((long long)nx * ny < (1LL << 20)) ? 64 : 0;
-        // whole launches of a tiled channel in a chunk by default
-        if (o.graph_steps == 0 && s->tile.h > 0 && !s->tile.whole) k = 2 * s->tile.h * std::max(1, 32 / s->tile.h);
+        // whole launches of a tiled channel in a chunk by default, an even number
+        // of them and 64 steps at least (fewer steps are launched one by one, also
+        // on a stream that is being captured, where no graph can be built)
+        if (o.graph_steps == 0 && s->tile.h > 0 && !s->tile.whole) k = 2 * s->tile.h * ((31 + s->tile.h) / s->tile.h);
         if (o.test_withhold_tile >= 0) k = 0;
         s->graph_steps = k + (k & 1);  // even: a chunk ends on the buffer it started from
     }
