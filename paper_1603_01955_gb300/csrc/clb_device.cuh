@@ -486,7 +486,7 @@ __device__ void gather_node(const SweepArgs& a, const KC<R>& c, const Field<T> f
     gather_node_at<R>(c, row_kind(y, a.ny),
                       [&](int i, int dy, int dx) -> R {
                           const T* p = f.base + i * f.plane + (long long)(y + dy) * a.pitch + a.xoff + (x + dx);
-                          return Codec<T>::dec(__ldg(p), c.isc);
+                          return Codec<T>::dec(*p, c.isc);
                       },
                       o);
 }
