@@ -81,13 +81,16 @@ template <class R> struct ParamSums {
     Acc<R> sv, sq, g, r;
 };
 
-// m = J_C(d)^T l for one node of a body-force channel (collide, MODE_PERIODIC)
-// and the node's parameter terms.  Capital names are adjoints.
+// What the reverse of a node's collision needs of its forward step (collide,
+// MODE_PERIODIC): velocity, moments, braces and kernels.  It does not depend on
+// the adjoint, so a walk can form it one step ahead.
+template <class R> struct Forward {
+    R rho, irho, jx, jy, ux, uy, ux2, uy2, uxy, kx, ky, nkxy, kxxy, kxyy, rf;
+    R t5u, t4, t5, t6, t7, g5, g6, g7, hp, hm;
+};
 template <class R>
-__device__ __forceinline__ void reverse_collide(const R (&d)[9], const R (&l)[9], R ref, const KC<R>& c, R (&m)[9],
-                                                ParamSums<R>& sum) {
-    const R h = R(0.5), q = R(0.25), two = R(2), third = R(1.0 / 3.0);
-    // forward: moments, braces and kernels
+__device__ __forceinline__ Forward<R> forward_of(const R (&d)[9], R ref, const KC<R>& c) {
+    const R h = R(0.5), two = R(2), third = R(1.0 / 3.0);
     const R a57 = d[5] + d[7], a68 = d[6] + d[8], p57 = d[5] - d[7], p86 = d[8] - d[6];
     const R nkxy = a68 - a57, kxxyy = a57 + a68, kxxy = p57 - p86, kxyy = p57 + p86;
     const R s13 = d[1] + d[3], s24 = d[2] + d[4];
@@ -107,6 +110,18 @@ __device__ __forceinline__ void reverse_collide(const R (&d)[9], const R (&l)[9]
     const R hp = R(1.5) * g3 + h * g4, hm = R(1.5) * g3 - h * g4;
     const R g6 = c.sq_4 * t6 - uy * hp - two * ux * g5;
     const R g7 = c.sq_4 * t7 - ux * hm - two * uy * g5;
+    return {rho, irho, jx, jy, ux, uy, ux2, uy2, uxy, kx, ky, nkxy, kxxy, kxyy, rf,
+            t5u, t4, t5, t6, t7, g5, g6, g7, hp, hm};
+}
+
+// m = J_C(d)^T l for one node of a body-force channel, from its forward_of(d),
+// and the node's parameter terms.  Capital names are adjoints.
+template <class R>
+__device__ __forceinline__ void reverse_collide(const Forward<R>& v, const R (&l)[9], const KC<R>& c, R (&m)[9],
+                                                ParamSums<R>& sum) {
+    const R h = R(0.5), q = R(0.25), two = R(2), fx = c.fx;
+    const auto [rho, irho, jx, jy, ux, uy, ux2, uy2, uxy, kx, ky, nkxy, kxxy, kxyy, rf,
+                t5u, t4, t5, t6, t7, g5, g6, g7, hp, hm] = v;
     // reverse of Eq. 6 and of the source (Eq. 9-10)
     const R A1 = l[1] + l[3], A2 = l[2] + l[4], D1 = l[1] - l[3], D2 = l[2] - l[4];
     const R S5 = l[5] + l[7], S6 = l[6] + l[8], E5 = l[7] - l[5], E6 = l[8] - l[6];
@@ -251,7 +266,7 @@ __device__ __forceinline__ void back_node(const R* f, const R* mu_next, const R*
         transpose_at(mu_next, push_of(k.nx, k.ny, x, y), k.r, k.rc, l);
     else
         for (int i = 0; i < 9; ++i) l[i] = lam[i * nn + node];
-    reverse_collide(fb, l, k.ref, k.c, m, sum);
+    reverse_collide(forward_of(fb, k.ref, k.c), l, k.c, m, sum);
     for (int i = 0; i < 9; ++i) mu[i * nn + node] = m[i];
     if (p.bottom) {
         wall_term(m[5], f[p.o[5]], f[p.wb[0]], sum.r);
@@ -330,10 +345,14 @@ __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* l
 // memory and block barriers only; the cluster barrier separates segments.
 // Other grids: every block of the cluster takes its share of the nodes of each
 // step, with a cluster barrier between steps (adj_cl_backward_kernel).
-// 4 x 64 nodes, FP32, per step: forward 0.36 us, backward 0.94 us (0.63 and
+// 4 x 64 nodes, FP32, per step: forward 0.34 us, backward 0.77 us (0.63 and
 // 6.46 us with the pulls worked out every step and J_C^T lambda formed by eleven
 // forward-mode columns over 16 blocks); both are bound by issue and latency in
-// their one block.  20 x 128 nodes, backward by a cluster: 3.2 us (31.4 us).
+// their one block.  A backward step of one warp per scheduler takes 0.58 us
+// (4 x 32), so its latency, not its issue, comes first: the forward part of
+// the next step, which does not wait for the adjoint, is formed beside the
+// reverse of this one (4 x 64 0.94 us and 4 x 32 0.72 us one after the other).
+// 20 x 128 nodes, backward by a cluster: 3.2 us (31.4 us).
 constexpr int kResThreads = 512;
 
 __device__ __forceinline__ double res_block_sum(double v, double* sh) {
@@ -494,8 +513,15 @@ __global__ void __launch_bounds__(kResThreads)
 #pragma unroll
                 for (int i = 4; i < 8; ++i) v.w[i] = e[i * nx];
         };
+        // one step's forward part is formed, and the next but one's values
+        // arrive, beside the reverse of this one
         Step cur, nxt;
-        if (live) load(len - 1, cur);
+        Forward<R> v{};
+        if (live) {
+            load(len - 1, cur);
+            v = forward_of(cur.fb, k.ref, k.c);
+            load(max(len - 2, 0), nxt);
+        }
         for (int j = len - 1; j >= 0; --j) {
             if (live) {
                 R l[9], m[9];
@@ -503,8 +529,10 @@ __global__ void __launch_bounds__(kResThreads)
                     for (int i = 0; i < 9; ++i) l[i] = lam_final[i * nn + node];
                 else
                     transpose_at(a, p, k.r, k.rc, l);
-                if (j > 0) load(j - 1, nxt);  // the next step's values arrive meanwhile
-                reverse_collide(cur.fb, l, k.ref, k.c, m, sum);
+                Step far;
+                load(max(j - 2, 0), far);
+                const Forward<R> next = forward_of(nxt.fb, k.ref, k.c);
+                reverse_collide(v, l, k.c, m, sum);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) b[i * nn + node] = m[i];
                 if (bottom) {
@@ -516,6 +544,8 @@ __global__ void __launch_bounds__(kResThreads)
                     wall_term(m[8], cur.w[6], cur.w[7], sum.r);
                 }
                 cur = nxt;
+                nxt = far;
+                v = next;
             }
             __syncthreads();
             R* q = a;
