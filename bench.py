@@ -34,15 +34,28 @@ METRIC = "D2Q9 CLB MLUPS and % HBM roofline, FP32-shifted vs FP64 at stated erro
 WORKLOAD = "pressure-driven microchannel L/H=100, Ny=256 x Nx=25601 (6.55M nodes), Kn_out=0.1, p_in/p_out=2.47"
 # sources of each sweep engine: a committed ncu summary is used only while the
 # hash of its engine's sources is the one it records
-DIRECT_SOURCES = ["paper_1603_01955_gb300/csrc/sweep.cu", "paper_1603_01955_gb300/csrc/clb_device.cuh",
-                  "paper_1603_01955_gb300/csrc/clb_internal.h"]
-TMA_SOURCES = DIRECT_SOURCES + ["paper_1603_01955_gb300/csrc/sweep_tma.cu",
-                                "paper_1603_01955_gb300/csrc/tma_common.cuh"]
+DIRECT_SOURCES = [f"paper_1603_01955_gb300/csrc/{p}" for p in ("sweep.cu", "clb_device.cuh", "pair.cuh", "clb_internal.h")]
+SOURCES = {"sweep": DIRECT_SOURCES,
+           "sweep_tma": DIRECT_SOURCES + [f"paper_1603_01955_gb300/csrc/{p}" for p in ("sweep_tma.cu", "tma_common.cuh")],
+           "march": DIRECT_SOURCES + [f"paper_1603_01955_gb300/csrc/{p}" for p in ("march.cu", "tma_common.cuh")]}
 
 
-def sweep_source_hash(pipeline: int = 2) -> str:
+def kernel_of(storage: str, requested: int, pipeline: int) -> str:
+    """The kernel that steps the benchmark channel: with the library's default
+    engine (requested 0) FP32 takes two steps per launch (march.cu; a step left
+    over is one TMA-staged sweep), else the sweep of clb_info's pipeline."""
+    if storage == "fp32s" and requested == 0:
+        return "march"
+    return "sweep" if pipeline <= 1 else "sweep_tma"
+
+
+def steps_per_launch(kernel: str) -> int:
+    return 2 if kernel == "march" else 1
+
+
+def sweep_source_hash(kernel: str = "sweep_tma") -> str:
     h = hashlib.sha256()
-    for p in (DIRECT_SOURCES if pipeline <= 1 else TMA_SOURCES):
+    for p in SOURCES[kernel]:
         with open(os.path.join(ROOT, p), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -56,10 +69,9 @@ def measured_peaks() -> tuple[float, str]:
         return 6800.0, "fallback"
 
 
-def profiled_value(storage: str, pipeline: int, key: str):
+def profiled_value(storage: str, kernel: str, key: str):
     """A figure (`key: value` line) from the committed ncu summary of that
-    engine, if it was taken on the current sweep sources (else None)."""
-    kernel = "sweep" if pipeline <= 1 else "sweep_tma"
+    kernel, if it was taken on the current sources (else None)."""
     path = os.path.join(ROOT, "profiles", f"{kernel}_{storage}_pressure_25601x256.md")
     try:
         text = open(path).read()
@@ -67,14 +79,14 @@ def profiled_value(storage: str, pipeline: int, key: str):
         return None
     m_hash = re.search(r"sweep_source_sha256:\s*([0-9a-f]+)", text)
     m_val = re.search(key + r":\s*([0-9.eE+]+)", text)
-    if not m_hash or not m_val or m_hash.group(1) != sweep_source_hash(pipeline):
+    if not m_hash or not m_val or m_hash.group(1) != sweep_source_hash(kernel):
         return None
     return float(m_val.group(1))
 
 
-def profiled_traffic(storage: str, pipeline: int):
-    """DRAM bytes per sweep launch (ncu summary), or None."""
-    return profiled_value(storage, pipeline, "traffic_bytes_per_launch")
+def profiled_traffic(storage: str, kernel: str):
+    """DRAM bytes per launch (ncu summary), or None."""
+    return profiled_value(storage, kernel, "traffic_bytes_per_launch")
 
 
 def flops_block(clb, results, nodes):
@@ -87,7 +99,7 @@ def flops_block(clb, results, nodes):
     peaks = {"f32": clb.clb_peak_fma(clb.CLB_FP32_SHIFTED), "f64": clb.clb_peak_fma(clb.CLB_FP64)}
     out = {"peak_tflops": {k: round(v, 3) for k, v in peaks.items()}, "peak_kind": "measured (clb_peak_fma)"}
     for storage, r in results.items():
-        ops = profiled_value(storage, r["pipeline"], "fp_ops_per_node")
+        ops = profiled_value(storage, r["kernel"], "fp_ops_per_node")
         prec = "f64" if storage == "fp64" else "f32"
         entry = {"precision": prec, "fp_ops_per_node": ops}
         if ops is not None:
@@ -248,13 +260,16 @@ def run_gpu(args):
         t_sweeps = e0.elapsed_time(e1) / 1e3
         t_obs = e1.elapsed_time(e2) / 1e3
         t_total = max_over_ranks(t_total, world, "cuda")
+        kernel = kernel_of(storage, args.pipeline, info["pipeline"])
         results[storage] = dict(
             pipeline=info["pipeline"],
+            kernel=kernel,
             mlups=replica_mlups(nodes, K, t_total, world),
             ms_per_step=t_total / K * 1e3,
             sweep_us=t_sweeps / K * 1e6,
             observables_us=t_obs * 1e6,
-            bytes_per_node=info["bytes_per_node"],
+            # per step: the populations once in and once out per launch
+            bytes_per_node=info["bytes_per_node"] / steps_per_launch(kernel),
             mass_flow=obs["mass_flow"],
             clocks=sampler.summary(),
         )
@@ -293,7 +308,7 @@ def run_gpu(args):
     f32 = results["fp32s"]
     peak, peak_kind = measured_peaks()
     achieved = f32["bytes_per_node"] * nodes / (f32["sweep_us"] * 1e-6) / 1e9
-    traffic = profiled_traffic("fp32s", f32["pipeline"])
+    traffic = profiled_traffic("fp32s", f32["kernel"])
     line = {
         "metric": METRIC,
         "value": round(f32["mlups"], 1),
@@ -311,10 +326,10 @@ def run_gpu(args):
             "workload": WORKLOAD,
             "nx": NX, "ny": NY, "kn_out": KN_OUT, "pressure_ratio": RATIO,
             "storage": "fp32s (deviations from w_i*rho_ref(x)), FP32 collide",
-            "step": "one fused stream-collide sweep per step; one FP64 observable reduction per timed region",
+            "step": "fused stream-collide, one or two steps per launch; one FP64 observable reduction per timed region",
             "l2": "no flush: each population buffer is 236 MB (FP32) / 472 MB (FP64), above the 129 MB L2",
             "parallelism": "replicas" if world > 1 else "single GPU",
-            "launch": engine_of(f32["pipeline"]),
+            "launch": engine_of(f32["kernel"], f32["pipeline"]),
         },
         "roofline": {
             "bound": "hbm",
@@ -323,9 +338,10 @@ def run_gpu(args):
             "unit": "GB/s",
             "frac": round(achieved / peak, 4),
             "traffic": traffic,
+            "steps_per_launch": steps_per_launch(f32["kernel"]),
             "peak_kind": peak_kind,
             "bytes_per_node": f32["bytes_per_node"],
-            "kernel": engine_of(f32["pipeline"])["kernel"],
+            "kernel": engine_of(f32["kernel"], f32["pipeline"])["kernel"],
         },
         "variants": variants_block(results, nodes, peak),
         "flops": flops_block(clb, results, nodes),
@@ -337,7 +353,8 @@ def run_gpu(args):
             "note": "per timed region: upload of the FP64 initial state from pinned host memory, K sweeps, "
                     "observables back to host; bytes per step = bytes per region / K",
         },
-        "gpu_launches": K + 1,  # K sweeps and one observable reduction
+        # K steps and one observable reduction
+        "gpu_launches": -(-K // steps_per_launch(f32["kernel"])) + 1,
         "clocks": clocks,
     }
     if not args.no_batch:
@@ -358,10 +375,10 @@ def adjoint_bench(clb, torch):
     ny = 64, Kn = 0.1, G = 1e-6, 20,000 FP32 steps with a checkpoint every 141
     steps.  Wall time of the checkpointed forward pass and of one backward
     pass (which recomputes every segment), per step, for the default engine
-    (the grid fits in shared memory: one block per pass) and for one launch
-    per step; and the device memory of the states they keep: ceil(N/C)
-    checkpoints + C + 1 segment states + 4 adjoint fields, each 9 nx ny FP32
-    values."""
+    (the grid fits in shared memory: one launch per pass) and for one launch
+    per step; and the device memory of the default engine's states: ceil(N/C)
+    checkpoints, two segments of C pulled states with 8 nx wall terms per step
+    and 3 adjoint fields, each state 9 nx ny FP32 values."""
     import math
 
     nx, ny, kn, g, n, every = 4, 64, 0.1, 1e-6, 20000, 141
@@ -383,8 +400,8 @@ def adjoint_bench(clb, torch):
         out[name] = {"forward_ms": round((t1 - t0) * 1e3, 2), "forward_us_per_step": round((t1 - t0) / n * 1e6, 3),
                      "backward_ms": round((t2 - t1) * 1e3, 2),
                      "backward_us_per_step": round((t2 - t1) / n * 1e6, 3), "q_norm": q, "dq_d_r_a_g": grad}
-    states = math.ceil(n / every) + every + 1 + 4
-    out.update(state_bytes=states * 9 * nx * ny * 4, states_kept=states)
+    states = math.ceil(n / every) + 2 * every + 3
+    out.update(state_bytes=(states * 9 * nx * ny + 16 * every * nx) * 4, states_kept=states)
     return out
 
 
@@ -499,8 +516,11 @@ def errors_vs_oracle(clb, variants, ref, steps):
 TMA_SHAPES = [(512, 2, 3), (128, 4, 2), (256, 4, 3)]
 
 
-def engine_of(pipeline: int) -> dict:
-    if pipeline <= 1:
+def engine_of(kernel: str, pipeline: int) -> dict:
+    if kernel == "march":
+        return {"pipeline": 0, "engine": "two steps per launch, rows of the middle time level in registers",
+                "strip_columns": 120, "kernel": "march_kernel"}
+    if kernel == "sweep":
         return {"pipeline": pipeline, "engine": "direct vector loads + warp shuffles", "vec": 4, "block_x": 128,
                 "kernel": "sweep_kernel<float, pressure, 4>"}
     nc, v, st = TMA_SHAPES[pipeline - 2]
@@ -518,7 +538,7 @@ def variants_block(results, nodes, peak):
     for storage, r in results.items():
         out[storage] = {"mlups": round(r["mlups"], 1), "mlups_sweeps": round(nodes / r["sweep_us"], 1),
                         "sweep_us": round(r["sweep_us"], 3), "observables_us": round(r["observables_us"], 1),
-                        "pipeline": r["pipeline"],
+                        "pipeline": r["pipeline"], "kernel": r["kernel"],
                         "bytes_per_node": r["bytes_per_node"],
                         "hbm_frac": round(r["bytes_per_node"] * nodes / (r["sweep_us"] * 1e-6) / 1e9 / peak, 4),
                         "mass_flow": r["mass_flow"], "clocks": r["clocks"]}
