@@ -334,10 +334,11 @@ typedef struct clb_adjoint clb_adjoint; /* opaque */
  * 2 C and 16 C where the allocator refuses that, or the former where it refuses
  * that too.  Synchronises.  nx * ny <= 2^22.
  * Engine: a grid whose two states fit in one block's shared memory
- * (2 * 9 nx ny elements <= about 200 KB: 2800 nodes in FP32) runs the
- * forward pass as one launch of one block and each backward pass as one
- * launch of a thread-block cluster (a pair of blocks for the FP32 grids above,
- * else 8 or 16); larger grids, or opts->pipeline = 1, use one launch per step.
+ * (2 * 9 nx ny elements <= about 200 KB: 2800 nodes in FP32), or an FP32 grid
+ * of at most 24,576 nodes, runs each pass as one launch: of one block or a pair
+ * of blocks for the smallest grids, else of a thread-block cluster of 16 blocks
+ * (8 where the device takes no more); larger grids, or opts->pipeline = 1, use
+ * one launch per step.
  * All give the same states; the sums of J and of the gradient are taken in
  * different orders. */
 clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, double g, int64_t nsteps,

@@ -14,7 +14,8 @@
 // P^T is a gather (each post-collision population is pulled by one node, or by
 // two wall nodes).  The forward keeps a checkpoint every C steps (C ~
 // sqrt(N)) and recomputes each segment before walking it backwards.
-// Parameter sums are FP64; states and adjoints are FP32 or FP64.
+// Parameter sums are FP64, or FP32 pairs of 48 bits; states and adjoints are FP32
+// or FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -209,11 +210,9 @@ constexpr int kAdjThreads = 128;
 // pulled by the node it streams to, or, at a wall, by the bounce-back and the
 // specular terms of Eq. 20 (two nodes of the wall row).  The offsets and
 // weights for one node, as Pull for the forward direction.
-__device__ __forceinline__ Pull push_of(int nx, int ny, int x, int y) {
+template <class At> __device__ __forceinline__ Pull push_with(int nx, int ny, int x, int y, At at) {
     Pull p;
-    const int nn = nx * ny;
     const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-    auto at = [&](int i, int yy, int xx) { return i * nn + yy * nx + xx; };
     p.top = y == ny - 1;
     p.bottom = y == 0;
     p.wb[0] = p.wb[1] = p.wt[0] = p.wt[1] = 0;
@@ -237,6 +236,9 @@ __device__ __forceinline__ Pull push_of(int nx, int ny, int x, int y) {
         p.wb[1] = at(5, y, xp);
     }
     return p;
+}
+__device__ __forceinline__ Pull push_of(int nx, int ny, int x, int y) {
+    return push_with(nx, ny, x, y, [&](int i, int yy, int xx) { return (i * ny + yy) * nx + xx; });
 }
 template <class R>
 __device__ __forceinline__ void transpose_at(const R* mu, const Pull& p, R r, R rc, R (&o)[9]) {
@@ -301,16 +303,17 @@ __global__ void __launch_bounds__(kAdjThreads)
     }
 }
 
-// One node's term of J = (1/nx) sum u_x of the final post-collision state, and
+// One node's term of J = (1/nx) sum u_x of the final post-collision state (its
+// populations at f[at + i stride]), and
 // its lambda_N = dJ/df_N: u_x = sum_i e_ix f_i / rho - G/2, so
 // dJ/df_i = (e_ix - u_x - G/2) / (nx rho).
 template <class R>
-__device__ __forceinline__ double flow_term(const R* f, R* lam, int node, const AdjConst<R>& k) {
+__device__ __forceinline__ double flow_term(const R* f, int stride, int at, R* lam, int node, const AdjConst<R>& k) {
     const int nn = k.nx * k.ny;
     const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
     double rho = (double)k.ref, jx = 0;
     for (int i = 0; i < 9; ++i) {
-        const double v = (double)f[i * nn + node];
+        const double v = (double)f[i * stride + at];
         rho += v;
         jx += ex[i] * v;
     }
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* l
     const int nn = k.nx * k.ny;
     double js = 0;
     for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x)
-        js += flow_term(f, lam, node, k);
+        js += flow_term(f, nn, node, lam, node, k);
     js = block_sum(js, sh);
     if (threadIdx.x == 0) acc[3 * gridDim.x + blockIdx.x] = js;
 }
@@ -333,8 +336,8 @@ __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* l
 // ------------------------------------------------------ resident engine
 //
 // The whole checkpointed forward pass is one launch, of one block with block
-// barriers between the steps where two states fit in its shared memory, else
-// (FP32) of a thread-block cluster with cluster barriers; the backward walk
+// barriers between the steps for the smallest grids (block_nodes), else of a
+// thread-block cluster with cluster barriers; the backward walk
 // over every segment is one launch of a cluster.  The parameter sums stay per thread (in step
 // order) and are added by fixed trees at the end, so the gradient is the same
 // bit for bit on every run.
@@ -344,7 +347,9 @@ __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* l
 // the other walks the segment after it backwards, each with its state in shared
 // memory and block barriers only; the cluster barrier separates segments.
 // Other grids: every block of the cluster takes its share of the nodes of each
-// step, with a cluster barrier between steps (adj_cl_backward_kernel).
+// step, with a cluster barrier between steps: the states in the blocks' shared
+// memory where each thread has one node (adj_share_*_kernel), in L2 where there
+// are more (adj_cl_*_kernel).
 // 4 x 64 nodes, FP32, per step: forward 0.34 us, backward 0.77 us (0.63 and
 // 6.46 us with the pulls worked out every step and J_C^T lambda formed by eleven
 // forward-mode columns over 16 blocks); both are bound by issue and latency in
@@ -352,7 +357,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* l
 // (4 x 32), so its latency, not its issue, comes first: the forward part of
 // the next step, which does not wait for the adjoint, is formed beside the
 // reverse of this one (4 x 64 0.94 us and 4 x 32 0.72 us one after the other).
-// 20 x 128 nodes, backward by a cluster: 3.2 us (31.4 us).
+// 20 x 128 nodes, by a cluster: forward 1.16, backward 2.2 us (31.4 us).
 constexpr int kResThreads = 512;
 
 __device__ __forceinline__ double res_block_sum(double v, double* sh) {
@@ -368,20 +373,19 @@ __device__ __forceinline__ double res_block_sum(double v, double* sh) {
 }
 
 // Steps of the whole grid in shared memory, from copy s to copy o (then the
-// other way round), with the block's barrier after each.  ONE: at most one
-// node per thread, whose pull is worked out once.  Before each collision,
-// visit(node, pulled populations, pull, state) sees the node.
-template <bool ONE, class R, class V>
+// other way round), with the block's barrier after each; a node per thread, at
+// most, whose pull is worked out once.  Before each collision, visit(step,
+// pulled populations, pull, state) sees the node.
+template <class R, class V>
 __device__ __forceinline__ void res_steps(R*& s, R*& o, long long nsteps, const AdjConst<R>& k, V&& visit) {
-    const int nn = k.nx * k.ny, node1 = threadIdx.x;
-    Pull p1{};
-    if (ONE && node1 < nn) p1 = pull_of(k.nx, k.ny, node1 % k.nx, node1 / k.nx);
+    const int nn = k.nx * k.ny, node = threadIdx.x;
+    Pull p{};
+    if (node < nn) p = pull_of(k.nx, k.ny, node % k.nx, node / k.nx);
     for (long long t = 0; t < nsteps; ++t) {
-        for (int node = node1; node < nn; node += ONE ? nn : blockDim.x) {
-            const Pull p = ONE ? p1 : pull_of(k.nx, k.ny, node % k.nx, node / k.nx);
+        if (node < nn) {
             R d[9];
             gather_at(s, p, k.r, k.rc, d);
-            visit(t, node, d, p, s);
+            visit(t, d, p, s);
             collide<R, MODE_PERIODIC>(d, k.ref, k.c);
 #pragma unroll
             for (int i = 0; i < 9; ++i) o[i * nn + node] = d[i];
@@ -395,7 +399,7 @@ __device__ __forceinline__ void res_steps(R*& s, R*& o, long long nsteps, const 
 
 // Forward pass from f^eq(rho_out, 0): checkpoint s (the state at step s C)
 // into ckpt + s state_elems, then J and lambda_N (as adj_final_kernel).
-template <class R, bool ONE>
+template <class R>
 __global__ void __launch_bounds__(kResThreads)
     adj_res_forward_kernel(R* ckpt, size_t state_elems, int every, long long nsteps, R* lam_final, double* J,
                            AdjConst<R> k) {
@@ -409,10 +413,10 @@ __global__ void __launch_bounds__(kResThreads)
     for (long long t = 0; t < nsteps; t += every) {
         R* c = ckpt + (size_t)(t / every) * state_elems;
         for (int e = threadIdx.x; e < n9; e += blockDim.x) c[e] = a[e];
-        res_steps<ONE>(a, b, min((long long)every, nsteps - t), k, [](long long, int, const R*, const Pull&, const R*) {});
+        res_steps(a, b, min((long long)every, nsteps - t), k, [](long long, const R*, const Pull&, const R*) {});
     }
     double js = 0;
-    for (int node = threadIdx.x; node < nn; node += blockDim.x) js += flow_term(a, lam_final, node, k);
+    for (int node = threadIdx.x; node < nn; node += blockDim.x) js += flow_term(a, nn, node, lam_final, node, k);
     js = res_block_sum(js, red);
     if (threadIdx.x == 0) *J = js;
 }
@@ -472,10 +476,10 @@ __global__ void __launch_bounds__(kResThreads)
         for (int e = threadIdx.x; e < n9; e += blockDim.x) a[e] = c[e];
         __syncthreads();
         R* out = seg + (size_t)(s % bufs) * seg_elems;
-        res_steps<true>(a, b, length(s), k, [&](long long t, int n1, const R* d, const Pull& p, const R* f) {
+        res_steps(a, b, length(s), k, [&](long long t, const R* d, const Pull& p, const R* f) {
             R* w = out + (size_t)t * step_elems;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) w[i * nn + n1] = d[i];
+            for (int i = 0; i < 9; ++i) w[i * nn + node] = d[i];
             R* e = w + n9 + x;
             if (bottom) {
                 e[0] = f[p.o[5]];
@@ -578,8 +582,7 @@ __global__ void __launch_bounds__(kResThreads)
 }
 
 // One block's nodes of a cluster, dealt out by whole warps, one to each block
-// in turn: the FP64 pipe takes 64 cycles per warp and instruction however few
-// lanes are live, so the fewest warps per SM finish first.  each(node, x, y);
+// in turn.  each(node, x, y);
 // a block's threads cover its share in one round (ONE) or several.
 struct ClusterNodes {
     int first, step, nx, x, y;
@@ -627,7 +630,7 @@ __global__ void __launch_bounds__(kResThreads)
         b = q;
     }
     double js = 0;
-    mine.each(nn, [&](int node, int, int) { js += flow_term(a, lam_final, node, k); });
+    mine.each(nn, [&](int node, int, int) { js += flow_term(a, nn, node, lam_final, node, k); });
     js = res_block_sum(js, red);
     if (threadIdx.x == 0) part[rank] = js;
 }
@@ -685,6 +688,271 @@ __global__ void __launch_bounds__(kResThreads)
     write_sums(sum, k, red, part + rank * 3);
 }
 
+// Grids of a node per thread of a cluster: each block holds its share in shared
+// memory, the columns (or the rows) from rank W (rank H) on, W x H nodes of
+// every block but the last as [9][H][W], and reads the others' where they are,
+// through the cluster's shared memory.  A step's round trip through L2, with
+// the fence that must precede its barrier, is gone.
+struct Share {
+    int nx, ny, W, H, rank, x0, y0, w, h, lastx;
+    bool live;         // this thread has a node:
+    int at, x, y, node;  // its place in the block's state, and in the grid
+    __device__ Share(int rank_, int nx_, int ny_, int W_, int H_) : nx(nx_), ny(ny_), W(W_), H(H_), rank(rank_) {
+        x0 = W < nx ? rank * W : 0;
+        y0 = H < ny ? rank * H : 0;
+        const bool any = rank == 0 || W < nx || H < ny;
+        w = any ? max(0, min(W, nx - x0)) : 0;
+        h = any ? max(0, min(H, ny - y0)) : 0;
+        lastx = (nx - 1) / W;
+        live = (int)threadIdx.x < w * h;
+        const int ly = live ? (int)threadIdx.x / w : 0, lx = live ? (int)threadIdx.x - ly * w : 0;
+        at = ly * W + lx;
+        x = x0 + lx;
+        y = y0 + ly;
+        node = y * nx + x;
+    }
+    // byte address, in the cluster's shared memory, of population i at (xx, yy),
+    // a neighbour of one of this block's nodes, in the buffers that start at base
+    template <class R> __device__ __forceinline__ int address(unsigned base, int i, int yy, int xx) const {
+        int r = rank, lx = xx - x0, ly = yy - y0;
+        if (lx < 0 || lx >= w) {  // columns: the next block, or around the end
+            r = xx == x0 + w && xx != nx ? rank + 1 : xx == x0 - 1 ? rank - 1 : xx == 0 ? 0 : lastx;
+            lx = xx - r * W;
+        }
+        if (ly < 0 || ly >= h) {  // rows
+            r = ly < 0 ? rank - 1 : rank + 1;
+            ly = yy - r * H;
+        }
+        unsigned to;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(base), "r"(r));
+        return (int)(to + (unsigned)(((i * H + ly) * W + lx) * (int)sizeof(R)));
+    }
+};
+
+__device__ __forceinline__ float ld_cluster(int a, float) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ double ld_cluster(int a, double) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    return v;
+}
+// The two halves of cluster_barrier, for what is in shared memory.
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// pull_of and gather_at, transpose_at, through addresses of the cluster's
+// shared memory (of buffer 0; off: of another).
+template <class At> __device__ __forceinline__ Pull pull_with(int nx, int ny, int x, int y, At at) {
+    Pull p;
+    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+    p.bottom = y == 0;
+    p.top = y == ny - 1;
+    p.wb[0] = p.wb[1] = p.wt[0] = p.wt[1] = 0;
+    p.o[0] = at(0, y, x);
+    p.o[1] = at(1, y, xm);
+    p.o[3] = at(3, y, xp);
+    p.o[2] = p.bottom ? at(4, y, x) : at(2, y - 1, x);
+    p.o[5] = p.bottom ? at(7, y, x) : at(5, y - 1, xm);
+    p.o[6] = p.bottom ? at(8, y, x) : at(6, y - 1, xp);
+    if (p.bottom) {
+        p.wb[0] = at(8, y, xm);
+        p.wb[1] = at(7, y, xp);
+    }
+    p.o[4] = p.top ? at(2, y, x) : at(4, y + 1, x);
+    p.o[7] = p.top ? at(5, y, x) : at(7, y + 1, xp);
+    p.o[8] = p.top ? at(6, y, x) : at(8, y + 1, xm);
+    if (p.top) {
+        p.wt[0] = at(6, y, xp);
+        p.wt[1] = at(5, y, xm);
+    }
+    return p;
+}
+template <class R> __device__ __forceinline__ void gather_cluster(const Pull& p, int off, R r, R rc, R (&f)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = ld_cluster(p.o[i] + off, R());
+    if (p.bottom) {
+        f[5] = ln::fma(r, f[5], ln::mul(rc, ld_cluster(p.wb[0] + off, R())));
+        f[6] = ln::fma(r, f[6], ln::mul(rc, ld_cluster(p.wb[1] + off, R())));
+    }
+    if (p.top) {
+        f[7] = ln::fma(r, f[7], ln::mul(rc, ld_cluster(p.wt[0] + off, R())));
+        f[8] = ln::fma(r, f[8], ln::mul(rc, ld_cluster(p.wt[1] + off, R())));
+    }
+}
+template <class R> __device__ __forceinline__ void transpose_cluster(const Pull& p, int off, R r, R rc, R (&o)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) o[i] = ld_cluster(p.o[i] + off, R());
+    if (p.top) {
+        o[5] = r * o[5] + rc * ld_cluster(p.wt[0] + off, R());
+        o[6] = r * o[6] + rc * ld_cluster(p.wt[1] + off, R());
+    }
+    if (p.bottom) {
+        o[7] = r * o[7] + rc * ld_cluster(p.wb[0] + off, R());
+        o[8] = r * o[8] + rc * ld_cluster(p.wb[1] + off, R());
+    }
+}
+
+// Threads of a block.  168 registers hold what the walk keeps from step to step;
+// with 448 threads and 128 registers it spills (20 x 128 2.52 us per backward
+// step against 2.19).  us per step forward + backward, against the round trip
+// through L2: 20 x 128 1.16 + 2.19, 1.93 + 3.22; 100 x 50 1.39 + 3.63, 2.17 +
+// 3.77; 75 x 80 1.22 + 3.22, 2.33 + 4.18; FP64 4 x 64 5.71 + 15.2, 6.07 + 15.8.
+// With several nodes per thread the addresses cost more than the round trip
+// (128 x 192 6.0 + 13.4 in shared memory; L2 see kClusterNodes).
+constexpr int kShareThreads = 384;
+
+// The forward pass, two copies of each block's share.  J's sums per block go to
+// part[rank].
+template <class R>
+__global__ void __launch_bounds__(kShareThreads)
+    adj_share_forward_kernel(R* ckpt, size_t state_elems, int every, long long nsteps, R* lam_final, double* part, int W,
+                             int H, AdjConst<R> k) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ double red[kResThreads];
+    const int nx = k.nx, ny = k.ny, nn = nx * ny, ws = W * H, bytes = 9 * ws * (int)sizeof(R);
+    const Share q(cluster_rank(), nx, ny, W, H);
+    const unsigned base = (unsigned)__cvta_generic_to_shared(sm_raw);
+    R* const s = reinterpret_cast<R*>(sm_raw);
+    Pull p{};
+    if (q.live) {  // zero deviations
+        for (int i = 0; i < 9; ++i) s[i * ws + q.at] = ckpt[i * nn + q.node] = R(0);
+        p = pull_with(nx, ny, q.x, q.y, [&](int i, int yy, int xx) { return q.template address<R>(base, i, yy, xx); });
+    }
+    int cur = 0;  // the copy that holds the state
+    cluster_arrive();
+    cluster_wait();
+    for (long long t = 0; t < nsteps; ++t) {
+        R d[9];
+        if (q.live) {
+            gather_cluster(p, cur * bytes, k.r, k.rc, d);
+            collide<R, MODE_PERIODIC>(d, k.ref, k.c);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) s[((cur ^ 1) * 9 + i) * ws + q.at] = d[i];
+        }
+        cluster_arrive();
+        if (q.live && (t + 1) % every == 0 && t + 1 < nsteps) {
+            R* c = ckpt + (size_t)((t + 1) / every) * state_elems;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) c[i * nn + q.node] = d[i];
+        }
+        cluster_wait();
+        cur ^= 1;
+    }
+    const double js = q.live ? flow_term(s + cur * 9 * ws, ws, q.at, lam_final, q.node, k) : 0.0;
+    const double sum = res_block_sum(js, red);
+    if (threadIdx.x == 0) part[q.rank] = sum;
+}
+
+// The backward walk: recompute the segment's states from its checkpoint, every
+// state also written to `seg`; then per step mu_t = J_C^T lambda_{t+1} with
+// lambda_{t+1} = P^T mu_{t+1} gathered from the blocks' shared memory (lambda_N
+// itself for the first step), one cluster barrier per step.  The state at t
+// comes from `seg` (L2): its pulls are loaded a step ahead, and in FP32 the
+// collision's forward part is formed while the barrier is on its way.  Three
+// buffers: mu of the last step, and the two that the recomputation, then the
+// walk, alternate with.  Every block runs the same loop counts, so every
+// barrier is reached by all of them.  Each block's parameter sums go to
+// part[rank * 3 + 0..2], added on the host in rank order.
+template <class R>
+__global__ void __launch_bounds__(kShareThreads)
+    adj_share_backward_kernel(const R* ckpt, R* seg, size_t state_elems, int every, long long nsteps, const R* lam_final,
+                              double* part, int W, int H, AdjConst<R> k) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ double red[kResThreads];
+    constexpr bool kEarly = std::is_same<R, float>::value;
+    const int nx = k.nx, ny = k.ny, nn = nx * ny, ws = W * H, bytes = 9 * ws * (int)sizeof(R);
+    const Share q(cluster_rank(), nx, ny, W, H);
+    const unsigned base = (unsigned)__cvta_generic_to_shared(sm_raw);
+    R* const s = reinterpret_cast<R*>(sm_raw);
+    auto addr = [&](int i, int yy, int xx) { return q.template address<R>(base, i, yy, xx); };
+    ParamSums<R> sum;
+    int last = 0, u = 1, v = 2;  // buffers: mu_{t+1}, and two to work in
+    const long long nseg = (nsteps + every - 1) / every;
+    for (long long sg = nseg - 1; sg >= 0; --sg) {
+        const int len = (int)min((long long)every, nsteps - sg * every);
+        const R* c = ckpt + (size_t)sg * state_elems;
+        if (q.live)
+            for (int i = 0; i < 9; ++i) s[(u * 9 + i) * ws + q.at] = seg[i * nn + q.node] = c[i * nn + q.node];
+        {
+            Pull p{};
+            if (q.live) p = pull_with(nx, ny, q.x, q.y, addr);
+            for (int j = 1; j < len; ++j) {
+                cluster_arrive();
+                cluster_wait();
+                if (q.live) {
+                    R* to = seg + (size_t)j * state_elems;
+                    R d[9];
+                    gather_cluster(p, u * bytes, k.r, k.rc, d);
+                    collide<R, MODE_PERIODIC>(d, k.ref, k.c);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) s[(v * 9 + i) * ws + q.at] = to[i * nn + q.node] = d[i];
+                }
+                const int o = u;
+                u = v;
+                v = o;
+            }
+        }
+        cluster_barrier();  // the segment's states are in global memory
+        Pull pf{}, pm{};  // pulls of the state, of mu
+        Forward<R> fw{};
+        if (q.live) {
+            pf = pull_of(nx, ny, q.x, q.y);
+            pm = push_with(nx, ny, q.x, q.y, addr);
+            if (kEarly) {
+                R fb[9];
+                gather_at(seg + (size_t)(len - 1) * state_elems, pf, k.r, k.rc, fb);
+                fw = forward_of(fb, k.ref, k.c);
+            }
+        }
+        for (int j = len - 1; j >= 0; --j) {
+            const R* f = seg + (size_t)j * state_elems;
+            R next[9], m[9];  // the pulls of step j - 1; mu_t
+            if (q.live) {
+                if (kEarly) {
+                    gather_at(f - (j > 0 ? state_elems : 0), pf, k.r, k.rc, next);
+                } else {
+                    gather_at(f, pf, k.r, k.rc, next);
+                    fw = forward_of(next, k.ref, k.c);
+                }
+                R l[9];
+                if (sg == nseg - 1 && j == len - 1)
+                    for (int i = 0; i < 9; ++i) l[i] = lam_final[i * nn + q.node];
+                else
+                    transpose_cluster(pm, last * bytes, k.r, k.rc, l);
+                reverse_collide(fw, l, k.c, m, sum);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) s[(u * 9 + i) * ws + q.at] = m[i];
+            }
+            cluster_arrive();
+            if (q.live) {
+                if (pf.bottom) {
+                    wall_term(m[5], f[pf.o[5]], f[pf.wb[0]], sum.r);
+                    wall_term(m[6], f[pf.o[6]], f[pf.wb[1]], sum.r);
+                }
+                if (pf.top) {
+                    wall_term(m[7], f[pf.o[7]], f[pf.wt[0]], sum.r);
+                    wall_term(m[8], f[pf.o[8]], f[pf.wt[1]], sum.r);
+                }
+                if (kEarly) fw = forward_of(next, k.ref, k.c);
+            }
+            cluster_wait();
+            const int o = last;
+            last = u;
+            u = o;
+        }
+    }
+    write_sums(sum, k, red, part + q.rank * 3);
+}
+
 // Shared memory of the resident forward kernel: two states and the block sum.
 size_t res_smem(int nx, int ny, size_t elem) {
     return ((2 * 9 * (size_t)nx * ny * elem + 15) / 16) * 16 + kResThreads * sizeof(double);
@@ -692,18 +960,19 @@ size_t res_smem(int nx, int ny, size_t elem) {
 // Threads of a resident block: one node each, by whole warps.
 int res_threads(int nx, int ny) { return std::min(kResThreads, (nx * ny + 31) / 32 * 32); }
 constexpr size_t kResSmemCap = 200 * 1024;
-// Largest FP32 grid of the cluster kernels, whose 16 blocks cost 0.3 us per
-// thousand nodes and step beyond 8192; one launch per step costs 5 us forward
+// Largest FP32 grid of the cluster kernels (with the states in L2, as below),
+// whose 16 blocks cost 0.3 us per thousand nodes and step beyond 8192; one launch per step costs 5 us forward
 // and 12 us backward whatever the grid.  Measured, us per step forward +
 // backward, cluster / launches: 100 x 50 2.3 + 3.8 / 4.8 + 12.3; 160 x 100
 // 3.9 + 7.0 / 5.2 + 12.4; 200 x 160 6.1 + 11.6 / 6.1 + 12.6; 320 x 200
 // 9.6 + 20.9 / 5.8 + 14.6.
 constexpr int kClusterNodes = 24576;
 // Nodes up to which the forward pass of a resident grid stays in one block.
-// FP32: 10 x 100 1.5 us per step there, 15 x 100 2.1, 20 x 128 3.3 (cluster 1.7).
+// FP32, one node per thread: 20 x 25 0.63 us per step there (cluster 25 x 41 0.91);
+// with two, 10 x 100 1.42.
 // FP64, bound by the FP64 pipe: 4 x 64 12.4 us there, 6.5 us in a cluster (one
 // warp per SM), where 4 x 32 takes as long.
-int block_nodes(size_t elem) { return elem == 8 ? 128 : 1024; }
+int block_nodes(size_t elem) { return elem == 8 ? 128 : kResThreads; }
 
 }  // namespace
 
@@ -812,6 +1081,38 @@ int cl_threads(const clb_adjoint* h, int cl) {
     return std::min(kResThreads, 32 * std::max(1, (warps + cl - 1) / cl));
 }
 
+// How a cluster of cl blocks shares a grid of a node per thread (one false:
+// there are more): by rows, whose nodes are next to each other in global
+// memory, or by columns where that makes a node per thread of it, or leaves a
+// share smaller by a fifth or more.  us per step forward + backward, by rows and
+// by columns: 64 x 64 1.20 + 2.62, 1.42 + 3.66; 100 x 50 (400 nodes by rows, two
+// per thread) 2.11 + 4.24, 1.60 + 3.95.
+struct Shares {
+    int W, H, threads;
+    bool one;
+    size_t state_bytes;
+};
+Shares shares_of(const clb_adjoint* h, int cl) {
+    const int w = (h->nx + cl - 1) / cl, r = (h->ny + cl - 1) / cl;
+    const long long by_columns = (long long)w * h->ny, by_rows = (long long)r * h->nx;
+    const bool columns = by_columns < by_rows && (by_rows > kShareThreads || 5 * by_columns <= 4 * by_rows);
+    Shares q;
+    q.W = columns ? w : h->nx;
+    q.H = columns ? h->ny : r;
+    const long long nodes = columns ? by_columns : by_rows;
+    q.one = nodes <= kShareThreads;
+    q.threads = (int)std::min<long long>(kShareThreads, (nodes + 31) / 32 * 32);
+    q.state_bytes = (size_t)9 * nodes * h->elem;
+    return q;
+}
+template <class K, class... A>
+cudaError_t launch_shares(K kern, int cl, const Shares& q, int copies, cudaStream_t st, A... args) {
+    const size_t smem = copies * q.state_bytes;
+    cudaError_t e = set_res_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    return launch_cluster(kern, cl, q.threads, smem, st, args...);
+}
+
 // Run launch(cl) with the largest cluster the device takes (16 blocks, else
 // the portable 8).
 template <class F> cudaError_t with_cluster(clb_adjoint* h, F&& launch) {
@@ -829,20 +1130,27 @@ template <class F> cudaError_t with_cluster(clb_adjoint* h, F&& launch) {
 
 // The forward pass in one block, or in one cluster (resident engine).
 template <class R> cudaError_t forward_resident(clb_adjoint* h) {
-    const size_t smem = res_smem(h->nx, h->ny, sizeof(R));
     int sums = 1;
     cudaError_t e;
-    if (smem <= kResSmemCap && h->nx * h->ny <= block_nodes(sizeof(R))) {
-        auto kern = h->nx * h->ny <= kResThreads ? adj_res_forward_kernel<R, true> : adj_res_forward_kernel<R, false>;
-        e = set_res_smem(kern, smem);
+    if (h->nx * h->ny <= block_nodes(sizeof(R))) {
+        const size_t smem = res_smem(h->nx, h->ny, sizeof(R));
+        e = set_res_smem(adj_res_forward_kernel<R>, smem);
         if (e != cudaSuccess) return e;
-        kern<<<1, res_threads(h->nx, h->ny), smem, h->stream>>>(
+        adj_res_forward_kernel<R><<<1, res_threads(h->nx, h->ny), smem, h->stream>>>(
             static_cast<R*>(h->ckpt), h->state_elems, h->every, (long long)h->nsteps, static_cast<R*>(h->lam_final),
             h->acc, kconst<R>(h));
         e = cudaGetLastError();
     } else {
         e = with_cluster(h, [&](int cl) {
-            return launch_cluster(adj_cl_forward_kernel<R>, cl, cl_threads(h, cl), 0, h->stream,
+            const Shares q = shares_of(h, cl);
+            if (q.one)
+                return launch_shares(adj_share_forward_kernel<R>, cl, q, 2, h->stream, static_cast<R*>(h->ckpt),
+                                     h->state_elems, h->every, (long long)h->nsteps, static_cast<R*>(h->lam_final),
+                                     h->acc, q.W, q.H, kconst<R>(h));
+            if constexpr (std::is_same<R, double>::value)
+                return cudaErrorInvalidValue;  // resident FP64 grids have a node per thread of 8 blocks
+            else
+                return launch_cluster(adj_cl_forward_kernel<R>, cl, cl_threads(h, cl), 0, h->stream,
                                   static_cast<R*>(h->ckpt), static_cast<R*>(h->seg), h->state_elems, h->every,
                                   (long long)h->nsteps, static_cast<R*>(h->lam_final), h->acc, kconst<R>(h));
         });
@@ -858,7 +1166,15 @@ template <class R> cudaError_t forward_resident(clb_adjoint* h) {
 }
 
 template <class R> cudaError_t launch_cl_backward(clb_adjoint* h, int cl) {
-    return launch_cluster(adj_cl_backward_kernel<R>, cl, cl_threads(h, cl), 0, h->stream, static_cast<const R*>(h->ckpt),
+    const Shares q = shares_of(h, cl);
+    if (q.one)
+        return launch_shares(adj_share_backward_kernel<R>, cl, q, 3, h->stream, static_cast<const R*>(h->ckpt),
+                             static_cast<R*>(h->seg), h->state_elems, h->every, (long long)h->nsteps,
+                             static_cast<const R*>(h->lam_final), h->acc, q.W, q.H, kconst<R>(h));
+    if constexpr (std::is_same<R, double>::value)
+        return cudaErrorInvalidValue;  // as in forward_resident
+    else
+        return launch_cluster(adj_cl_backward_kernel<R>, cl, cl_threads(h, cl), 0, h->stream, static_cast<const R*>(h->ckpt),
                           static_cast<R*>(h->seg), h->state_elems, h->every, (long long)h->nsteps,
                           static_cast<const R*>(h->lam_final), static_cast<R*>(h->mu0), static_cast<R*>(h->mu),
                           h->acc, kconst<R>(h));

@@ -28,7 +28,12 @@ def clb():
     ("fp32s", 1e-5, 16, 32, 200, 17), ("fp32s", 1e-5, 19, 27, 200, 17), ("fp32s", 1e-5, 25, 41, 200, 400),
     ("fp32s", 1e-5, 91, 90, 120, 11), ("fp32s", 1e-5, 128, 192, 60, 0), ("fp32s", 1e-5, 173, 143, 60, 0),
     ("fp64", 1e-12, 1, 1, 60, 7), ("fp64", 1e-12, 4, 32, 200, 17), ("fp64", 1e-12, 3, 43, 200, 17),
-    ("fp64", 1e-12, 31, 45, 60, 0), ("fp64", 1e-12, 40, 40, 40, 0)])
+    ("fp64", 1e-12, 31, 45, 60, 0), ("fp64", 1e-12, 40, 40, 40, 0),
+    # a cluster with a node per thread: full blocks, one node more per block than
+    # that, shares by columns, blocks left without nodes, single rows and columns
+    ("fp32s", 1e-5, 96, 64, 60, 0), ("fp32s", 1e-5, 97, 64, 60, 0), ("fp32s", 1e-5, 100, 50, 90, 13),
+    ("fp32s", 1e-5, 40, 33, 90, 1), ("fp32s", 1e-5, 6000, 1, 60, 0), ("fp32s", 1e-5, 1, 600, 90, 7),
+    ("fp32s", 1e-5, 3000, 2, 60, 0), ("fp64", 1e-12, 100, 12, 40, 7), ("fp64", 1e-12, 300, 1, 40, 40)])
 def test_engines_match_one_launch_per_step(clb, storage, tol, nx, ny, n, every):
     out = []
     for pipeline in (0, 1):
