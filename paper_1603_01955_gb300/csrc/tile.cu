@@ -444,17 +444,33 @@ template <class F> cudaError_t with_tile(int storage, int mode, const TilePlan& 
 // against 2.9 us; 801 x 8 periodic 0.68 against 2.6; 4 x 32 in one block 0.33
 // against 2.8; 6401 x 64 stays with the direct sweep (7.2 against 6.3 us).
 // FP64 (pair.cuh), in the same way: a step costs 1.2 us, 3.2 us with the end of
-// a pressure channel, and 10 ns per node; the direct sweep 4.6 or 8.2 us and
+// a pressure channel, and 10 ns per node; the direct sweep 3.7 or 8.2 us and
 // 0.048 ns per node.  801 x 8 pressure: 5.3 us per step, against 8.1; periodic
-// 2.8 against 4.6; 4 x 32 in one block 2.0 against 4.7; 2101 x 33 stays with the
+// 2.8 against 3.8; 4 x 32 in one block 2.0 against 4.7; 2101 x 33 stays with the
 // direct sweep (9.0 against 7.7).
+//
+// That model ranks the step counts; it is short on tall narrow tiles, whose
+// copies and passes cost more.  So the plan found is kept only where a second
+// estimate, fitted to 194 timed plans of 8 to 300 rows and 15,000 to 320,000
+// nodes (within 8 % in the mean, 26 % at most), is below the direct sweep's by
+// 5 %.  us per step, tiles and direct: 3026 x 76 BF16 periodic 5.45 / 3.28, 1428 x
+// 49 3.12 / 2.60, 7187 x 32 3.89 / 3.78, 5882 x 17 2.49 / 2.83; pressure 909 x 110
+// 4.49 / 4.04, 3026 x 76 4.40 / 4.48, 3061 x 49 3.16 / 4.08.
+struct Fit {  // us, thousands of nodes
+    double step, node, launch, copy;   // a step, each node of the block; a launch, each node its block moves
+    double flat, direct, direct_node;  // the direct sweep: at least flat
+};
+constexpr Fit kFit[2][2] = {  // [16 bits][pressure]
+    {{0.234, 0.835, 3.465, 3.475, 2.36, 1.843, 0.0083}, {0.802, 0.718, 4.381, 1.945, 2.96, 2.069, 0.0108}},
+    {{0.095, 0.958, 6.911, 4.113, 2.73, 2.006, 0.0071}, {1.023, 0.260, 2.841, 4.272, 3.99, 3.409, 0.0056}}};
+
 TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_cap) {
     TilePlan best;
     if (ny > kTileThreads || sms < 1) return best;
     const size_t elem = storage == 0 ? 8 : storage == 1 ? 4 : 2, relem = storage == 0 ? 8 : 4;
     const int cs = ny | 1;
     const bool f64 = storage == 0, press = mode == MODE_PRESSURE;
-    double best_t = 0.9 * (f64 ? (press ? 8200.0 : 4600.0) + 0.048 * nx * ny : 2500.0 + 0.01 * nx * ny);
+    double best_t = 0.9 * (f64 ? (press ? 8200.0 : 3700.0) + 0.048 * nx * ny : 2500.0 + 0.01 * nx * ny);
     auto consider = [&](int blocks, int h, bool whole) {
         const int w = (nx + blocks - 1) / blocks, cols = whole ? nx : w + 2 * h;
         const bool big = (size_t)cols * cs > plane_of(elem, false);
@@ -490,6 +506,13 @@ TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_
     const int blocks = std::max(1, std::min(sms, nx / 3));
     if (nx / blocks >= 3)
         for (int h = 1; h <= 32; ++h) consider(blocks, h, false);
+    if (best.h > 0 && !best.whole && !f64) {
+        const int w = (nx + best.blocks - 1) / best.blocks;
+        const Fit& f = kFit[elem == 2][press];
+        const double tall = 1e-3 * ny, nodes = 1e-3 * nx * ny;
+        const double tiles = f.step + f.node * tall * (w + best.h) + (f.launch + f.copy * tall * (2 * w + 2 * best.h)) / best.h;
+        if (tiles > 0.95 * std::max(f.flat, f.direct + f.direct_node * nodes)) return TilePlan{};
+    }
     return best;
 }
 
