@@ -852,12 +852,16 @@ __global__ void __launch_bounds__(kShareThreads)
     if (threadIdx.x == 0) part[q.rank] = sum;
 }
 
-// The backward walk: recompute the segment's states from its checkpoint, every
-// state also written to `seg`; then per step mu_t = J_C^T lambda_{t+1} with
-// lambda_{t+1} = P^T mu_{t+1} gathered from the blocks' shared memory (lambda_N
-// itself for the first step), one cluster barrier per step.  The state at t
-// comes from `seg` (L2): its pulls are loaded a step ahead, and in FP32 the
-// collision's forward part is formed while the barrier is on its way.  Three
+// The backward walk: recompute the segment's states from its checkpoint, which
+// is its state 0, every later one also written to `seg`; then per step mu_t =
+// J_C^T lambda_{t+1} with lambda_{t+1} = P^T mu_{t+1} gathered from the blocks'
+// shared memory (lambda_N itself for the first step), one cluster barrier per
+// step.  The state at t comes from L2: its pulls are loaded a step ahead, and in
+// FP32 the collision's forward part is formed while the barrier is on its way.
+// The wall terms read it after the barrier's arrival, when another thread may
+// already be in the next segment: state 0 is therefore read where nothing writes
+// it (the checkpoint), and a later one is rewritten only beyond a further barrier
+// (that of a later step of the walk), which its readers arrive at first.  Three
 // buffers: mu of the last step, and the two that the recomputation, then the
 // walk, alternate with.  Every block runs the same loop counts, so every
 // barrier is reached by all of them.  Each block's parameter sums go to
@@ -881,7 +885,8 @@ __global__ void __launch_bounds__(kShareThreads)
         const int len = (int)min((long long)every, nsteps - sg * every);
         const R* c = ckpt + (size_t)sg * state_elems;
         if (q.live)
-            for (int i = 0; i < 9; ++i) s[(u * 9 + i) * ws + q.at] = seg[i * nn + q.node] = c[i * nn + q.node];
+            for (int i = 0; i < 9; ++i) s[(u * 9 + i) * ws + q.at] = c[i * nn + q.node];
+        auto state = [&](int j) { return j > 0 ? seg + (size_t)j * state_elems : c; };
         {
             Pull p{};
             if (q.live) p = pull_with(nx, ny, q.x, q.y, addr);
@@ -909,16 +914,16 @@ __global__ void __launch_bounds__(kShareThreads)
             pm = push_with(nx, ny, q.x, q.y, addr);
             if (kEarly) {
                 R fb[9];
-                gather_at(seg + (size_t)(len - 1) * state_elems, pf, k.r, k.rc, fb);
+                gather_at(state(len - 1), pf, k.r, k.rc, fb);
                 fw = forward_of(fb, k.ref, k.c);
             }
         }
         for (int j = len - 1; j >= 0; --j) {
-            const R* f = seg + (size_t)j * state_elems;
+            const R* f = state(j);
             R next[9], m[9];  // the pulls of step j - 1; mu_t
             if (q.live) {
                 if (kEarly) {
-                    gather_at(f - (j > 0 ? state_elems : 0), pf, k.r, k.rc, next);
+                    gather_at(state(max(j - 1, 0)), pf, k.r, k.rc, next);
                 } else {
                     gather_at(f, pf, k.r, k.rc, next);
                     fw = forward_of(next, k.ref, k.c);
