@@ -67,8 +67,9 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) march_kernel(const Sweep
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const float* __restrict__ fin = static_cast<const float*>(a.fin);
-    float* __restrict__ fout = static_cast<float*>(a.fout);
+    // no __restrict__: the previous launch may still write the input when this one starts
+    const float* fin = static_cast<const float*>(a.fin);
+    float* fout = static_cast<float*>(a.fout);
     float4* const slot = reinterpret_cast<float4*>(smem) + warp * kAhead * 9 * 32 + lane;  // [stage][population][lane]
 
     const bool edge = (int)blockIdx.x < p.edge_blocks;

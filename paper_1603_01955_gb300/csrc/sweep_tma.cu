@@ -46,8 +46,9 @@ __global__ void __launch_bounds__(NC + 32, MB) sweep_tma_kernel(const SweepArgs 
     uint64_t* empty = full + S;
     __shared__ int abort_flag;
     __shared__ int2 stage_tile[S];  // (row, column tile) of each stage; row -1: no more tiles
-    const T* __restrict__ fin = static_cast<const T*>(a.fin);
-    T* __restrict__ fout = static_cast<T*>(a.fout);
+    // no __restrict__: the previous launch may still write the input when this one starts
+    const T* fin = static_cast<const T*>(a.fin);
+    T* fout = static_cast<T*>(a.fout);
     const KC<R>& c = a.ks;  // constants in the units of the stored values
     const Field<T> src{fin, a.plane};
 

@@ -73,7 +73,9 @@ __global__ void __launch_bounds__(kTileThreads + kEndThreads, 1)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    const T* __restrict__ fin = static_cast<const T*>(a.fin);
+    // No __restrict__ on the input: the previous launch may still write it when this
+    // one starts, so it must not be read through the read-only path.
+    const T* fin = static_cast<const T*>(a.fin);
     T* __restrict__ fout = static_cast<T*>(a.fout);
     // Global <-> shared copies: a thread moves four columns of a row at once
     // (16 bytes of FP32), a warp 8 such vectors of 4 rows, which keeps both the
