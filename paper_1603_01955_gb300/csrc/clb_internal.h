@@ -136,8 +136,8 @@ struct TilePlan {
 };
 constexpr int kTileMaxSteps = 4096;  // steps per launch of a whole channel in one block
 TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_cap);
-// Allow the plan's shared memory on the current device.
-cudaError_t tile_opt_in(int storage, int mode, const TilePlan& p);
+// Allow the plan's kernel smem_cap bytes of shared memory, on the current device.
+cudaError_t tile_opt_in(int storage, int mode, const TilePlan& p, size_t smem_cap);
 cudaError_t launch_tiles(int storage, int mode, const TilePlan& p, const SweepArgs& a, int nsteps, cudaStream_t st);
 
 }  // namespace clb

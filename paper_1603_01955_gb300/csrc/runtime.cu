@@ -728,8 +728,9 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
         const int mode = drive == CLB_DRIVE_PRESSURE ? MODE_PRESSURE : MODE_PERIODIC;
         int cap = 0;
         cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        s->tile = plan_tiles(o.storage, mode, nx, ny, sms, (size_t)std::max(cap, 0));
-        if (s->tile.h > 0 && tile_opt_in(o.storage, mode, s->tile) != cudaSuccess) {
+        cap = std::max(cap, 0);
+        s->tile = plan_tiles(o.storage, mode, nx, ny, sms, (size_t)cap);
+        if (s->tile.h > 0 && tile_opt_in(o.storage, mode, s->tile, (size_t)cap) != cudaSuccess) {
             cudaGetLastError();
             s->tile = TilePlan{};
         }

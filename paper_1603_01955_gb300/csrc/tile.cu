@@ -518,9 +518,11 @@ TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_
     return best;
 }
 
-cudaError_t tile_opt_in(int storage, int mode, const TilePlan& p) {
+// The limit belongs to the kernel, not to a channel: it is always the cap that
+// plans are made under, so that no channel's plan lowers it below another's.
+cudaError_t tile_opt_in(int storage, int mode, const TilePlan& p, size_t smem_cap) {
     return with_tile(storage, mode, p, [&](auto kern) {
-        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cap);
     });
 }
 

@@ -1,0 +1,47 @@
+"""Objects of different sizes held together: the shared memory a kernel may take
+is set per kernel and process, so creating or running one object must not take
+it from another, in either order of creation, launched one by one or replayed,
+or from another thread.  Every object gives the bits it gives alone."""
+import threading
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def clb():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1603_01955_gb300.clb as clb
+
+    return clb
+
+
+SIZES = {"pressure": [(801, 8), (1601, 16), (2101, 21), (2401, 24), (401, 8)],
+         "body_force": [(801, 8), (1601, 16), (701, 5), (4, 32), (40, 31)]}
+
+
+@pytest.mark.parametrize("storage", ["fp32s", "fp16s", "bf16s", "fp64"])
+@pytest.mark.parametrize("drive", ["pressure", "body_force"])
+def test_tiled_channels_together(clb, storage, drive):
+    def make(nx, ny, **kw):
+        return clb.Channel(nx, ny, 0.2, drive=drive, drive_value=1.8 if drive == "pressure" else 1e-5, storage=storage, **kw)
+
+    want = {}
+    for size in SIZES[drive]:
+        ch = make(*size, pipeline=1)
+        ch.step(213)
+        want[size] = ch.state()
+        ch.close()
+    for order in (SIZES[drive], SIZES[drive][::-1]):
+        chans = {size: make(*size) for size in order}
+        for n in (3, 200, 10):
+            for ch in chans.values():
+                ch.step(n)
+        for size, ch in chans.items():
+            np.testing.assert_array_equal(ch.state(), want[size])
+            ch.close()
