@@ -465,12 +465,14 @@ bool plan_sched(const clb_batch* b, int npt, int packed, int block_min, BatchSch
     }
 }
 
-template <class T> cudaError_t set_smem_limit(size_t bytes) {
+// The limit belongs to the kernel, not to a schedule: always the cap that
+// schedules are made under, so that no trial or other batch lowers it.
+template <class T> cudaError_t set_smem_limit() {
     cudaError_t e = cudaSuccess;
     const void* ks[] = {(const void*)batch_kernel<T, 1>, (const void*)batch_kernel<T, 2>,
                         (const void*)batch_kernel<T, 4>, (const void*)batch_kernel<T, 8>};
     for (const void* k : ks) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
         if (e != cudaSuccess) break;
     }
     if (e == cudaSuccess)
@@ -500,7 +502,7 @@ clb_status make_sched(clb_batch* b, int npt, int packed, int block_min, BatchSch
     if (e == cudaSuccess) e = cudaMemcpyAsync(m + oo, order.data(), bo, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(m + os, slots.data(), bs, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
-        e = b->storage == CLB_FP64 ? set_smem_limit<double>(t.smem) : set_smem_limit<float>(t.smem);
+        e = b->storage == CLB_FP64 ? set_smem_limit<double>() : set_smem_limit<float>();
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // the host vectors go out of scope
     if (e != cudaSuccess) {
         b->dfree(t.mem);

@@ -45,3 +45,37 @@ def test_tiled_channels_together(clb, storage, drive):
         for size, ch in chans.items():
             np.testing.assert_array_equal(ch.state(), want[size])
             ch.close()
+
+
+@pytest.mark.parametrize("storage", ["fp32s", "fp64"])
+def test_batches_together(clb, storage):
+    shapes = [dict(nx=[4] * 3, ny=[300, 128, 40], kn=[0.1, 0.3, 1.0]), dict(nx=[4, 3], ny=[32, 16], kn=[0.2, 0.5]),
+              dict(nx=[4] * 2, ny=[200, 64], kn=[0.05, 2.0])]
+
+    def make(schedule, **kw):
+        b = clb.Batch(kw["nx"], kw["ny"], kw["kn"], g=1e-5, storage=storage)
+        if schedule:
+            b.set_schedule(*schedule)
+        else:
+            b.tune()
+        return b
+
+    def states(b):
+        out = [b.state(k) for k in range(b.n)]
+        b.close()
+        return out
+
+    want = []
+    for kw in shapes:
+        b = make((8, 0), **kw)
+        b.step(613)
+        want.append(states(b))
+    for schedule in ((8, 0), (4, 1), None):
+        for order in ((0, 1, 2), (2, 1, 0)):
+            batches = {k: make(schedule, **shapes[k]) for k in order}
+            for n in (3, 600, 10):
+                for b in batches.values():
+                    b.step(n)
+            for k, b in batches.items():
+                for x, y in zip(states(b), want[k]):
+                    np.testing.assert_array_equal(x, y)
