@@ -1053,8 +1053,11 @@ cudaError_t sum_partials(clb_adjoint* h, int rows, double* out) {
     return cudaSuccess;
 }
 
-template <class K> cudaError_t set_res_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// Allow a kernel the shared memory of the largest resident grid.  The limit
+// belongs to the kernel for the whole process: one value for every grid, so that
+// no other handle (or thread) lowers it between this and the launch.
+template <class K> cudaError_t opt_in(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemCap);
 }
 
 // Launch fn's kernel with its arguments as one cluster of `cl` blocks (more
@@ -1112,10 +1115,9 @@ Shares shares_of(const clb_adjoint* h, int cl) {
 }
 template <class K, class... A>
 cudaError_t launch_shares(K kern, int cl, const Shares& q, int copies, cudaStream_t st, A... args) {
-    const size_t smem = copies * q.state_bytes;
-    cudaError_t e = set_res_smem(kern, smem);
+    cudaError_t e = opt_in(kern);
     if (e != cudaSuccess) return e;
-    return launch_cluster(kern, cl, q.threads, smem, st, args...);
+    return launch_cluster(kern, cl, q.threads, copies * q.state_bytes, st, args...);
 }
 
 // Run launch(cl) with the largest cluster the device takes (16 blocks, else
@@ -1139,7 +1141,7 @@ template <class R> cudaError_t forward_resident(clb_adjoint* h) {
     cudaError_t e;
     if (h->nx * h->ny <= block_nodes(sizeof(R))) {
         const size_t smem = res_smem(h->nx, h->ny, sizeof(R));
-        e = set_res_smem(adj_res_forward_kernel<R>, smem);
+        e = opt_in(adj_res_forward_kernel<R>);
         if (e != cudaSuccess) return e;
         adj_res_forward_kernel<R><<<1, res_threads(h->nx, h->ny), smem, h->stream>>>(
             static_cast<R*>(h->ckpt), h->state_elems, h->every, (long long)h->nsteps, static_cast<R*>(h->lam_final),
@@ -1187,10 +1189,9 @@ template <class R> cudaError_t launch_cl_backward(clb_adjoint* h, int cl) {
 
 cudaError_t launch_pair_backward(clb_adjoint* h) {
     using R = float;
-    const size_t smem = 2 * h->state_elems * sizeof(R);
-    cudaError_t e = set_res_smem(adj_pair_backward_kernel<R>, smem);
+    cudaError_t e = opt_in(adj_pair_backward_kernel<R>);
     if (e != cudaSuccess) return e;
-    return launch_cluster(adj_pair_backward_kernel<R>, 2, res_threads(h->nx, h->ny), smem, h->stream,
+    return launch_cluster(adj_pair_backward_kernel<R>, 2, res_threads(h->nx, h->ny), 2 * h->state_elems * sizeof(R), h->stream,
                           static_cast<const R*>(h->ckpt), static_cast<R*>(h->seg), h->state_elems, h->every,
                           (long long)h->nsteps, h->seg_bufs, static_cast<const R*>(h->lam_final), h->acc, kconst<R>(h));
 }

@@ -79,3 +79,32 @@ def test_batches_together(clb, storage):
             for k, b in batches.items():
                 for x, y in zip(states(b), want[k]):
                     np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("storage,grids", [("fp32s", [(4, 64), (2, 9), (100, 50), (20, 40)]),
+                                           ("fp64", [(31, 45), (4, 64), (2, 9), (12, 30)])])
+def test_gradients_in_threads(clb, storage, grids):
+    def gradient(nx, ny):
+        fg = clb.FlowGradient(nx, ny, 0.3, 2.0, 0.8, 2e-5, 40, storage=storage)
+        out = (fg.J, *fg.grad())
+        fg.close()
+        return out
+
+    want = {g: gradient(*g) for g in grids}
+    wrong = []
+
+    def work(g):
+        try:
+            for _ in range(60):
+                got = gradient(*g)
+                if got != want[g]:
+                    wrong.append((g, got))
+        except Exception as e:  # noqa: BLE001 - reported below, in the test's own thread
+            wrong.append((g, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(g,)) for g in grids]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong, wrong[:4]
