@@ -23,11 +23,18 @@ namespace {
 
 thread_local char g_err[512] = "";
 
+// A CUDA error that is reported is not left as the runtime's last error, where
+// the check after another object's next launch would find it.
+void clear_reported(int st) {
+    if (st == CLB_ECUDA) cudaGetLastError();
+}
+
 clb_status fail(clb_status st, const char* fmt, ...) {
     va_list ap;
     va_start(ap, fmt);
     vsnprintf(g_err, sizeof g_err, fmt, ap);
     va_end(ap);
+    clear_reported(st);
     return st;
 }
 
@@ -594,6 +601,7 @@ int set_error(int st, const char* fmt, ...) {
     va_start(ap, fmt);
     vsnprintf(g_err, sizeof g_err, fmt, ap);
     va_end(ap);
+    clear_reported(st);
     return st;
 }
 
