@@ -127,6 +127,13 @@ CLB_HD P twice(P a) { return {fmul(2.0f, a.h), fmul(2.0f, a.l)}; }
 CLB_HD P scale(P a, float p2) { return {fmul(p2, a.h), fmul(p2, a.l)}; }  // by a power of two
 // constants (folded at compile time, or on the host)
 CLB_HD constexpr P pair_of(double v) { return {(float)v, (float)(v - (double)(float)v)}; }
+// Whether a density can be split and collided with (2^-12 to 2^30), by its high
+// word: a NaN, an infinity, a negative or another number out of FP32's range
+// would come out of split as some finite one.
+CLB_HD bool in_range(double v) {
+    const uint32_t m = hi(v);
+    return m >= (1011u << 20) && m < (1053u << 20);
+}
 // 1 / a for normalised a > 0: the FP32 reciprocal y and its correction
 // y (e + e^2), e = 1 - a y formed with fused multiply-adds.
 CLB_HD P inv(P a) {
