@@ -342,8 +342,8 @@ __device__ __forceinline__ void collide(L (&d)[9], L ref, const KC<R>& c, const 
 }
 
 // The FP64 collision of a node (densities, R = 0): in FP32 pairs where the
-// node is near enough to equilibrium (pair.cuh) and the density that sets its
-// Knudsen number can be a pair, else in plain FP64, out of
+// node is near enough to equilibrium (pair.cuh) and the launch's constants and
+// the density that sets its Knudsen number can be pairs, else in plain FP64, out of
 // line: few nodes take it, and its registers are not the fast path's.
 template <int MODE>
 __device__ __noinline__ void collide_plain64(double* f, const KC<double>* c, const double* rho_kn) {
@@ -360,7 +360,7 @@ __device__ __forceinline__ void collide64(double (&f)[9], const KC<double>& c, c
     float R;
     pr::P d[9], o[9];
     const bool near = pr::deviations(f, R, d);
-    if (near && (MODE != MODE_PRESSURE || !rho_kn || pr::in_range(*rho_kn))) {
+    if (near && kp.fits && (MODE != MODE_PRESSURE || !rho_kn || pr::in_range(*rho_kn))) {
         pr::P kn{0.0f, 0.0f};
         if (MODE == MODE_PRESSURE && rho_kn) kn = pr::split(*rho_kn);
         pr::collide<MODE == MODE_PERIODIC>(R, d, kp, MODE == MODE_PRESSURE && rho_kn ? &kn : nullptr, o);

@@ -177,7 +177,13 @@ struct Const {
     P s3_12, s8_4, sv_4, sq_4;  // as KC
     P A, B, A316, CA;
     P fx, hfx;
+    bool fits;                  // every constant is one that pairs can hold (fits)
 };
+// Whether a launch constant can be held and multiplied as a pair: below 2^40 in
+// magnitude, so that the largest product of the rates, B (A316 B), stays in
+// FP32's range and the reciprocal's.  (ny Kn from 1.3e-13 to 8e11; beyond, every
+// node takes the plain FP64 collision.)
+CLB_HD bool fits(double v) { return v < 0x1p40 && v > -0x1p40; }
 
 // Densities of the populations f: R, about their sum (to 2^-19, each taken by
 // the high word of its double), the deviations d from w_i R as pairs

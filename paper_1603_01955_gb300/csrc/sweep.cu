@@ -392,7 +392,9 @@ void derive_constants(SweepArgs& a) {
     const KC<double>& d = a.kd;
     a.kp = pr::Const{pr::pair_of(d.s3_12), pr::pair_of(d.s8_4), pr::pair_of(d.sv_4), pr::pair_of(d.sq_4),
                      pr::pair_of(d.A),     pr::pair_of(d.B),    pr::pair_of(d.A316), pr::pair_of(d.CA),
-                     pr::pair_of(d.fx),    pr::pair_of(d.hfx)};
+                     pr::pair_of(d.fx),    pr::pair_of(d.hfx),  true};
+    for (double v : {d.s3_12, d.s8_4, d.sv_4, d.sq_4, d.A, d.B, d.A316, d.CA, d.fx, d.hfx})
+        a.kp.fits = a.kp.fits && pr::fits(v);
     // densities scale, 1/densities scale inversely, rates and velocities do not
     KC<float>& k = a.ks;
     k = a.kf;

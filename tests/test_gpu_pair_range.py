@@ -46,3 +46,35 @@ def test_centre_density_out_of_range(clb, oracle_mod, pipeline, bad):
         rest = np.arange(nx) != xb
         assert (np.abs(got - want)[:, far][:, :, rest] / np.abs(want[:, far][:, :, rest])).max() <= 1e-12
     ch.close()
+
+
+@pytest.mark.parametrize("pipeline", [0, 1])
+@pytest.mark.parametrize("kn", [1e-45, 1e-39, 1e-14, 1e12, 1e38, 1e100])
+def test_rate_constants_out_of_range(clb, oracle_mod, pipeline, kn):
+    """Knudsen numbers whose constants no FP32 number holds, and those beside them."""
+    nx, ny = 40, 9
+    ch = clb.Channel(nx, ny, kn, drive="pressure", drive_value=1.5, storage="fp64", pipeline=pipeline)
+    orc = oracle_mod.OracleSim(oracle_mod.OracleParams(nx=nx, ny=ny, pressure=True, kn=kn, rho_in=1.5))
+    f = inputs.perturb(inputs.rng(4), orc.state(), 0.01)
+    ch.set_state(f)
+    orc.set_state(f)
+    ch.step(2)
+    orc.step(2)
+    want = orc.state()
+    assert (np.abs(ch.state() - want) / np.abs(want)).max() <= 1e-12
+    ch.close()
+
+
+def test_force_out_of_range(clb, oracle_mod):
+    """A body force beyond FP32: the step that has it is the plain one, without an infinity."""
+    ch = clb.Channel(6, 9, 0.2, drive="body_force", drive_value=1e60, storage="fp64")
+    orc = oracle_mod.OracleSim(oracle_mod.OracleParams(nx=6, ny=9, kn=0.2, gx=1e60))
+    f = inputs.perturb(inputs.rng(5), orc.state(), 0.01)
+    ch.set_state(f)
+    orc.set_state(f)
+    ch.step(1)
+    orc.step(1)
+    got, want = ch.state(), orc.state()
+    assert np.isfinite(want).all()
+    assert np.abs(got - want).max() <= 1e-12 * np.abs(want).max()
+    ch.close()

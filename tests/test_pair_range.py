@@ -38,3 +38,46 @@ def compile_and_run(source, tmp_path):
 def test_densities_taken(tmp_path):
     r = compile_and_run(SOURCE, tmp_path)
     assert r.returncode == 0, r.stdout
+
+
+CONSTANTS = r"""
+#include <cstdio>
+#include <cmath>
+#include <initializer_list>
+#include "pair.cuh"
+using namespace clb::pr;
+// The increments with launch constants from every Knudsen number whose constants
+// fit, against long double: the rates' error, 2^-40 at the most, times the
+// deviations, plus that of the pairs.
+int main() {
+    int taken = 0;
+    for (double e = -320; e < 308; e += 0.25) {
+        const double kn = pow(10.0, e), ny = 8, A = sqrt(6 / M_PI) * ny * kn, B = 2 * kn, A316 = 3 / (16 * A), CA = M_PI * 0.55 / 4 * A;
+        bool fit = true;
+        for (double v : {A, B, A316, CA}) fit = fit && fits(v);
+        if (e >= -12 && e <= 10 && !fit) return printf("refused %g\n", kn), 1;
+        if (!fit) continue;
+        ++taken;
+        const Const c{pair_of(1.1 / 12), pair_of(0.3), {}, {}, pair_of(A), pair_of(B), pair_of(A316), pair_of(CA), {}, {}, true};
+        double f[9];
+        float R;
+        P d[9], o[9];
+        for (int i = 0; i < 9; ++i) f[i] = (i == 0 ? 4. / 9 : i < 5 ? 1. / 9 : 1. / 36) * (1 + 1e-3 * ((7 * i) % 5 - 2));
+        if (!deviations(f, R, d)) return printf("state\n"), 1;
+        collide<false>(R, d, c, nullptr, o);
+        // g5 = s_v/4 (rho ux uy - kxy) is the part of o[5] + o[7] - o[6] - o[8] (Eq. 6)
+        long double rho = 0, jx = 0, jy = 0, kxy = 0;
+        const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+        for (int i = 0; i < 9; ++i) rho += f[i], jx += ex[i] * (long double)f[i], jy += ey[i] * (long double)f[i], kxy += ex[i] * ey[i] * (long double)f[i];
+        const long double q = rho + B, sv = q / (q / 2 + A), g5 = sv / 4 * (jx * jy / rho - kxy);
+        const long double got = ((long double)o[5].h + o[5].l + o[7].h + o[7].l - o[6].h - o[6].l - o[8].h - o[8].l) / 4;
+        if (!(fabsl(got - g5) <= 1e-3L * 0x1p-40L)) return printf("kn %g: %Lg against %Lg\n", kn, got, g5), 1;
+    }
+    return taken < 80;
+}
+"""
+
+
+def test_constants_taken(tmp_path):
+    r = compile_and_run(CONSTANTS, tmp_path)
+    assert r.returncode == 0, r.stdout
