@@ -1378,6 +1378,8 @@ clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, do
     h->lam_final = h->dalloc(sb);
     h->mu = h->dalloc(sb);
     h->nb = blocks_for((size_t)nx * ny, kAdjThreads);
+    h->acc = static_cast<double*>(h->dalloc(std::max<size_t>(4 * (size_t)h->nb, 3 * kClusterMax) * sizeof(double)));
+    // (the segment comes last: it may take less where memory is short)
     // one launch per pass, unless opts->pipeline asks for one launch per step
     // (1), while that is faster than filling the GPU in each of two or three
     // launches per step: see the rule's figures at kClusterNodes
@@ -1398,7 +1400,6 @@ clb_status clb_adjoint_forward(int nx, int ny, double kn, double a, double r, do
         h->pair = h->seg != nullptr;
     }
     if (!h->seg) h->seg = h->dalloc(sb * (h->every + 1));
-    h->acc = static_cast<double*>(h->dalloc(std::max<size_t>(4 * (size_t)h->nb, 3 * kClusterMax) * sizeof(double)));
     if (!h->ckpt || !h->seg || !h->mu0 || !h->lam_final || !h->mu || !h->acc) {
         clb_adjoint_destroy(h);
         return (clb_status)set_error(CLB_ENOMEM, "clb_adjoint_forward: device allocation failed");
