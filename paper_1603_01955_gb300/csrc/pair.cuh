@@ -9,9 +9,11 @@
 // and delta is computed from d in pairs h + l of FP32 numbers (48 bits; the
 // sums and products of Dekker and Knuth), at about 900 FP32 operations.  d and
 // delta are small where the flow is near equilibrium, so their 48 bits reach
-// below the last bit of f; a node where they are not small (|d_i| > R/64, a
-// flow above about a twentieth of the lattice speed, or R not within 2^+-30)
-// takes the plain FP64 collision instead.
+// below the last bit of f; a node where they are not small (|d_i| > R/32, a flow
+// above 0.094 lattice speeds, or R not from 2^-12 to 2^30) takes the plain FP64
+// collision instead.  The bound is where the populations' rms error is still
+// below the plain collision's (velocities to 0.08: 4.9e-17 against 6.1e-17; 0.12,
+// beyond it: 8e-17).
 //
 // Measured, 25601 x 256 pressure channel: 316 us per sweep against 1455 us;
 // the 18 FP64 operations alone take 225 us.  rms error of a population after
@@ -206,9 +208,9 @@ CLB_HD bool deviations(const double (&f)[9], float& R, P (&d)[9]) {
         big = m > big ? m : big;
         d[i] = split(v, m);
     }
-    // |d| <= R/64, compared as high words: a NaN, an infinity or a value out
+    // |d| <= R/32, compared as high words: a NaN, an infinity or a value out
     // of FP32's range (whose R means nothing) is above
-    return R >= 2.4414062e-4f && R <= 1.07e9f && big < rh - (6u << 20);
+    return R >= 2.4414062e-4f && R <= 1.07e9f && big < rh - (5u << 20);
 }
 
 struct Moments {
