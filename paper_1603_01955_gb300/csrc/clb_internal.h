@@ -125,6 +125,7 @@ cudaError_t launch_march(int sms, const SweepArgs& a, cudaStream_t st);
 // Several steps per launch of a small channel held in shared memory (tile.cu).
 struct TilePlan {
     int h = 0;            // steps per launch at most (0: no plan)
+    int few = 1;          // a launch of fewer steps is left to the direct sweep
     bool whole = false;   // one block holds the whole channel (no halo)
     bool pack = false;    // two nodes per packed FP32 collision
     bool big = false;     // the larger constant plane in shared memory

@@ -853,7 +853,7 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
 }
 
 // One launch from buffer `cur`: a sweep (direct or TMA engine), or `steps`
-// steps of the channel in tiles.
+// steps of the channel in tiles (at least TilePlan::few).
 static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur, int steps = 1) {
     const size_t rc_side = (size_t)2 * s->rc_stride * (s->storage == CLB_FP64 ? 8 : 4);
     a.fin = s->buf[cur];
@@ -862,7 +862,7 @@ static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur, in
     a.rc_out = static_cast<char*>(s->rc) + (cur ^ 1) * rc_side;
     a.tile_order = cur;  // alternate the TMA sweep's tile order with the buffers
     if (steps == 2 && s->march_sms) return launch_march(s->march_sms, a, s->stream);
-    if (s->tile.h > 0) return launch_tiles(s->storage, mode, s->tile, a, steps, s->stream);
+    if (s->tile.h > 0 && steps >= s->tile.few) return launch_tiles(s->storage, mode, s->tile, a, steps, s->stream);
     return s->pipeline >= 2 ? launch_sweep_tma(s->storage, mode, s->pipeline - 2, a, s->stream, s->sched, s->status)
                             : launch_sweep(s->storage, mode, s->vec, s->block_x, a, s->stream);
 }
@@ -876,7 +876,11 @@ static cudaError_t launch_steps(clb_sim* s, SweepArgs& a, int mode, int* cur, in
     if (even && launches % 2) ++launches;
     *done = 0;
     for (; launches > 0; --launches) {
-        const int64_t k = (n - *done + launches - 1) / launches;
+        int64_t k = (n - *done + launches - 1) / launches;
+        if (s->tile.h > 0 && k < s->tile.few && k > 1) {  // as that many sweeps
+            launches += k - 1;
+            k = 1;
+        }
         cudaError_t e = launch_single(s, a, mode, *cur, (int)k);
         if (e != cudaSuccess) return e;
         *cur ^= 1;

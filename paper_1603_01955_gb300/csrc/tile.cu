@@ -508,6 +508,14 @@ TilePlan plan_tiles(int storage, int mode, int nx, int ny, int sms, size_t smem_
     const int blocks = std::max(1, std::min(sms, nx / 3));
     if (nx / blocks >= 3)
         for (int h = 1; h <= 32; ++h) consider(blocks, h, false);
+    // One step alone is faster as a direct sweep (us per call, tiles and sweep: 801
+    // x 8 FP32 3.6 / 2.6, pressure 3.8 / 3.1; 2101 x 33 6.9 / 2.9; FP64 457 x 33
+    // pressure 9.6 / 8.2), but for low 16-bit pressure channels (801 x 8 FP16 3.9 /
+    // 4.3, 1601 x 16 4.3 / 4.3, 2101 x 21 4.9 / 4.4).  So are two where one block
+    // copies the channel in more than one round of rows in flight (4 x 32 FP32 6.8 /
+    // 5.3, FP16 10.7 / 6.0, FP64 11.5 / 9.6; 16 x 16, in one round, 4.2 / 4.6).
+    best.few = elem == 2 && press && !best.whole && ny <= 16 ? 1 : 2;
+    if (best.whole && 9 * ny > 9 * (best.threads / 8)) best.few = 3;  // 9 rows of 8 threads each in flight
     if (best.h > 0 && !best.whole && !f64) {
         const int w = (nx + best.blocks - 1) / best.blocks;
         const Fit& f = kFit[elem == 2][press];
