@@ -66,7 +66,13 @@ typedef enum {
 } clb_drive;
 
 typedef enum {
-    CLB_FP64 = 0,         /* populations stored and collided in FP64 (144 B per node update) */
+    /* Populations stored in FP64 (144 B per node update), moved by increments
+     * that are computed in pairs of FP32 numbers (48 bits) from FP64 deviations
+     * and are no less precise than plain FP64's; nodes that move at more than
+     * 0.094 lattice speeds or are otherwise far from equilibrium, and channels
+     * whose constants FP32 cannot hold, collide in plain FP64, which takes several
+     * times as long. */
+    CLB_FP64 = 0,
     CLB_FP32_SHIFTED = 1, /* FP32 deviations f - w_i rho_ref(x), FP32 collision (72 B) */
     CLB_FP16_SCALED = 2,  /* FP16 deviations times a field scale 2^14, FP32 collision (36 B) */
     CLB_BF16_SCALED = 3   /* BF16 deviations (scale 1), FP32 collision (36 B) */
@@ -100,8 +106,9 @@ typedef struct {
      * persistent grid.  With all of pipeline, vec and block_x 0, small
      * channels advance several steps per launch in shared memory and FP32
      * pressure channels of 500,000 nodes and at least 2000 columns two steps
-     * per launch; the engine named above then takes what is left over.  All
-     * give bit-identical results. */
+     * per launch; the engine named above then takes what is left over, and
+     * calls of one step (of two, where that is faster).  All give bit-identical
+     * results. */
     int pipeline;
     /* Local Knudsen number of a pressure channel (Sec. 3.2): 0 = from the
      * node's own pressure (default), 1 = from the centreline pressure p(x) of

@@ -52,7 +52,7 @@ template <typename R> struct Wt {
 };
 
 // FP32: the hardware reciprocal (PTX rcp.approx, within 1 ulp); its error is
-// far below the FP32 storage rounding.  FP64: the IEEE quotient.
+// far below the FP32 storage rounding.
 __device__ __forceinline__ float rcp(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -127,8 +127,7 @@ __device__ __forceinline__ void macro_dev(const R d[9], R& drho, R& jx, R& jy) {
 // gets the same bits whether it is collided alone (float, double) or together
 // with its neighbour in packed FP32 (float2: the f32x2 instructions of
 // sm_100-class GPUs add, multiply or fused-multiply-add both halves of a
-// register pair at once, each half rounded as the scalar operation).  Other
-// number types (the dual numbers of the adjoint) use their operators.
+// register pair at once, each half rounded as the scalar operation).
 namespace ln {
 __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
@@ -172,11 +171,6 @@ __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ float neg(float a) { return -a; }
 __device__ __forceinline__ double neg(double a) { return -a; }
 __device__ __forceinline__ float2 neg(float2 a) { return mul(a, make_float2(-1.0f, -1.0f)); }
-template <class L> __device__ __forceinline__ L neg(L a) { return -a; }
-template <class L> __device__ __forceinline__ L add(L a, L b) { return a + b; }
-template <class L> __device__ __forceinline__ L sub(L a, L b) { return a - b; }
-template <class L> __device__ __forceinline__ L mul(L a, L b) { return a * b; }
-template <class L> __device__ __forceinline__ L fma(L a, L b, L c) { return a * b + c; }
 // a scalar in every lane
 template <class L, class S> __device__ __forceinline__ L bc(S s) {
     if constexpr (std::is_same<L, float2>::value)

@@ -17,13 +17,15 @@
 // below and the row above its own at t+1, the outer lanes recompute their
 // neighbours' columns: 11 % of the collisions at 51 rows per segment.
 //
-// What bounds it: 42 bytes per node and step cross HBM at 5.9 TB/s, 0.86 of the
-// copy peak, and the warps issue at half rate.  8 warps per SM, not more: with
-// 12 the same bytes move at 5.0 TB/s and with 16 at 4.6, the more streams of
-// 480 bytes the worse, and at 16 the registers spill.  25601 x 256: 46.7 us per
-// step, against 72 us of the TMA-staged sweep.  16-bit storage gains nothing (46
-// against 41 us: as many instructions, half the bytes to save), nor do periodic
-// channels (71 against 72 us: a third more instructions for the body force).
+// What bounds it: the fixed latencies of the collision's dependent chain, with
+// two warps per scheduler (issue slots 45 % busy; 1.17 waiting warps per issued
+// instruction, 0.08 of them for loads).  HBM carries the 36 algorithmic bytes per
+// node and step at 0.73 of the copy peak.  8 warps per SM, not more: with 12 the
+// same bytes move more slowly, the more streams of 480 bytes the worse, and at 16
+// the registers spill.  25601 x 256: 47.8 us per step, against 71.6 us of the
+// TMA-staged sweep.  16-bit storage gains nothing (47.5 us with 12 warps, against
+// 40.8: as many instructions, half the bytes to save), nor do periodic channels
+// (71 against 72 us: a third more instructions for the body force).
 //
 // The arithmetic per node is that of sweep.cu, bit for bit.
 #include <algorithm>
@@ -345,8 +347,8 @@ cudaError_t launch_march(int sms, const SweepArgs& a, cudaStream_t st) {
     p.edges = std::min(p.strips, 3);
     p.groups = (p.strips - p.edges + kWarps - 1) / kWarps;
     // a wave of segments of one length, the edge strips' half as long, keeps
-    // neighbouring strips at the same rows, which HBM likes (25601 x 256: 46.7
-    // us per step, with equal shares 49.0); shares where whole segments would
+    // neighbouring strips at the same rows, which HBM likes (25601 x 256: with
+    // equal shares 1.05 times as long); shares where whole segments would
     // leave more than a fifth of the wave empty (80000 x 40: 35.6 and 24.8 us).
     // At least 4 rows each: every segment recomputes two.
     p.segs = (int)std::min(slots / (p.groups + 2.0 * p.edges / kWarps), std::max(1.0, ny / 4.0));

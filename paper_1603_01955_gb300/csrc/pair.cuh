@@ -11,15 +11,22 @@
 // delta are small where the flow is near equilibrium, so their 48 bits reach
 // below the last bit of f; a node where they are not small (|d_i| > R/32, a flow
 // above 0.094 lattice speeds, or R not from 2^-12 to 2^30) takes the plain FP64
-// collision instead.  The bound is where the populations' rms error is still
-// below the plain collision's (velocities to 0.08: 4.9e-17 against 6.1e-17; 0.12,
-// beyond it: 8e-17).
+// collision instead.  Up to that bound the populations' rms error stays below the
+// plain collision's; at twice the bound it would not (see below).
 //
 // Measured, 25601 x 256 pressure channel: 316 us per sweep against 1455 us;
 // the 18 FP64 operations alone take 225 us.  rms error of a population after
 // one collision, relative to the density, against long double: 8e-18 to 1.6e-17
-// for velocities of 1e-3 to 0.05, against 3.4e-17 of the plain form (whose
-// moments sum populations, not deviations); density and momentum as before.
+// for velocities of 1e-3 to 0.04 and 2.8e-17 at 0.08, against 3.4e-17 of the plain
+// form (whose moments sum populations, not deviations); 4.4e-17 at 0.12, beyond the
+// bound.  Density and momentum as before, 4 to 10 % more at non-equilibrium parts of
+// 1 %.  Whole runs end closer to long double than with the plain form: 4 x 32
+// periodic, 1000 steps, rms of the state 7.6e-17 against 3.1e-16.
+//
+// A flow beyond the bound pays for both forms.  us per step, against the plain
+// collision alone: 200 x 20 pressure at a velocity of 0.114 20.4 / 12.9, 457 x 33 at
+// 0.19 18.9 / 13.5, 300 x 128 at 0.33 23.1 / 21.0, 801 x 17 periodic at 0.21 10.3 /
+// 8.8; within it 200 x 20 at 0.053 5.9 / 13.0.
 //
 // Host compilers see the same arithmetic (no fused contraction), so that its
 // error can be measured there.

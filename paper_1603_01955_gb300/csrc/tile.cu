@@ -442,7 +442,7 @@ template <class F> cudaError_t with_tile(int storage, int mode, const TilePlan& 
 //   shrinking halo), and where the block holds the end of a pressure channel
 //   at least 1.05 us, the latency of rebuilding its end column;
 // - the direct sweep costs 2.5 us per step and 0.01 ns per node of the channel.
-// 1601 x 16 pressure FP32: w 11, h 9, expected 1.4, measured 1.25 us per step,
+// 1601 x 16 pressure FP32: w 11, h 24, expected 1.22, measured 1.36 us per step,
 // against 2.9 us; 801 x 8 periodic 0.68 against 2.6; 4 x 32 in one block 0.33
 // against 2.8; 6401 x 64 stays with the direct sweep (7.2 against 6.3 us).
 // FP64 (pair.cuh), in the same way: a step costs 1.2 us, 3.2 us with the end of
