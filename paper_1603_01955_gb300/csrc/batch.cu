@@ -202,29 +202,33 @@ __global__ void __launch_bounds__(512) batch_kernel(const BatchArgs a, const Sch
         for (int e = lt; e < 9 * nn; e += nth) g[e] = s[e];
 }
 
-// The same for one channel per block, one node per thread and two copies, where
-// every block has an SM to itself: the planes and the copies lie at constant
+// The same in FP32 for one channel per block, one node per thread and two copies,
+// where every block has an SM to itself: the planes and the copies lie at constant
 // distances, the steps are unrolled by two, and so every access to shared memory
 // is a register worked out once per launch and an immediate offset.  The largest
 // block is bound by issue (four warps per scheduler, 240 instructions per node
 // and step with addresses worked out at every access).  48 channels of 4 x 16 to
 // 4 x 128 nodes: 0.52 us per step against 0.558; two nodes per thread 0.63.
+// A launch costs 2 us more (its state is spread over the planes and gathered
+// again), so one of few steps takes batch_kernel: one channel of 4 x 32, us per
+// launch of 1, 20 and 40 steps 5.0, 9.1 and 13.1, here 6.9, 10.8 and 13.1; 48
+// channels 6.7, 17.1, 27.5 and 8.9, 17.2, 27.5.  FP64 gains nothing (48 channels
+// 6.0 us per step both ways) and loses where a warp is alone on its scheduler (4 x
+// 32: 1.95 against 2.8): two copies of the pair collision's code.
+constexpr int kOneSteps = 32;
 constexpr int kPlane = 512;  // elements of a population's plane
-template <class T> constexpr int kOneSmem = 2 * 9 * kPlane * (int)sizeof(T);
+constexpr int kOneSmem = 2 * 9 * kPlane * (int)sizeof(float);
 
-template <class T>
 __global__ void __launch_bounds__(kPlane) batch_one_kernel(const BatchArgs a, const SchedArgs sc, int nsteps) {
-    using R = T;
+    using R = float;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int k = sc.order[sc.groups[blockIdx.x].x];
     const BatchChannel ch = a.ch[k];
     const KC<R> c = kcs<R>(a)[k];
-    pr::Const kp{};
-    if (std::is_same<R, double>::value) kp = a.kp[k];
     const int nx = ch.nx, ny = ch.ny, nn = nx * ny, node = threadIdx.x;
     const R r = c.r, rc = c.rc, ref = c.ref0;
     R* const s = reinterpret_cast<R*>(smem_raw);
-    T* g = static_cast<T*>(a.state) + ch.offset;
+    R* g = static_cast<R*>(a.state) + ch.offset;
     auto spread = [&](int e) { return e + e / nn * (kPlane - nn); };  // of [9][nn] in planes of kPlane
     for (int e = threadIdx.x; e < 9 * nn; e += blockDim.x) s[spread(e)] = g[e];
     const bool live = node < nn;
@@ -245,10 +249,7 @@ __global__ void __launch_bounds__(kPlane) batch_one_kernel(const BatchArgs a, co
         if (live) {
             R f[9];
             gather_at(s + kFrom, p, r, rc, f);
-            if constexpr (std::is_same<R, double>::value)
-                collide64<MODE_PERIODIC>(f, c, kp);
-            else
-                collide<R, MODE_PERIODIC>(f, ref, c);
+            collide<R, MODE_PERIODIC>(f, ref, c);
 #pragma unroll
             for (int i = 0; i < 9; ++i) s[kTo + i * kPlane + node] = f[i];
         }
@@ -475,8 +476,6 @@ template <class T> cudaError_t set_smem_limit() {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
         if (e != cudaSuccess) break;
     }
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(batch_one_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOneSmem<T>);
     return e;
 }
 
@@ -492,7 +491,7 @@ clb_status make_sched(clb_batch* b, int npt, int packed, int block_min, BatchSch
     if (!plan_sched(b, npt, packed, block_min, t, groups, order, slots))
         return (clb_status)set_error(CLB_EINVAL, "clb_batch: schedule (%d nodes per thread, packed %d) does not fit",
                                      npt, packed);
-    t.one = npt == 1 && !packed && t.two_buffers && t.nblocks <= sms && t.block <= kPlane;
+    t.one = b->storage != CLB_FP64 && npt == 1 && !packed && t.two_buffers && t.nblocks <= sms && t.block <= kPlane;
     const size_t bg = groups.size() * sizeof(int2), bo = order.size() * sizeof(int), bs = slots.size() * sizeof(BatchSlot);
     const size_t og = 0, oo = (bg + 15) / 16 * 16, os = oo + (bo + 15) / 16 * 16;
     t.mem = b->dalloc(os + bs);
@@ -518,8 +517,8 @@ template <class T>
 cudaError_t launch_batch(clb_batch* b, const BatchSched& sc, void* state, int nsteps, cudaStream_t st) {
     BatchArgs a{state, b->dch, b->dkf, b->dkd, b->dkp};
     dim3 grid(sc.nblocks), blk(sc.block);
-    if (sc.one) {
-        batch_one_kernel<T><<<grid, blk, kOneSmem<T>, st>>>(a, sc.args, nsteps);
+    if (sc.one && nsteps >= kOneSteps) {
+        batch_one_kernel<<<grid, blk, kOneSmem, st>>>(a, sc.args, nsteps);
         return cudaGetLastError();
     }
     switch (sc.npt) {
