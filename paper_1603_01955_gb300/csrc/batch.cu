@@ -761,7 +761,7 @@ clb_status clb_batch_tune(clb_batch* b, int* block_out) {
                 continue;
             }
             err = cudaMemcpyAsync(scratch, b->state, b->total * b->elem, cudaMemcpyDeviceToDevice, b->stream);
-            if (err == cudaSuccess) err = launch(b, sc, scratch, 20, b->stream);  // warm-up
+            if (err == cudaSuccess) err = launch(b, sc, scratch, kOneSteps, b->stream);  // warm-up, of the kernel that is timed
             if (err == cudaSuccess) err = cudaEventRecord(e0, b->stream);
             if (err == cudaSuccess) err = launch(b, sc, scratch, trial_steps, b->stream);
             if (err == cudaSuccess) err = cudaEventRecord(e1, b->stream);
