@@ -311,8 +311,10 @@ clb_status clb_batch_schedule(const clb_batch* b, int* threads_per_block, int* n
 clb_status clb_batch_observables(clb_batch* b, clb_scalars* s);
 
 /* Channel k's populations as FP64 host arrays [9][ny][nx] (layout of
- * clb_get_state).  Synchronises; goes through the batch's pinned staging array
- * (72 bytes per node of its largest channel). */
+ * clb_get_state).  Synchronises; takes a transient device buffer, or, once that
+ * many calls have been made or are to be expected (58, the channels counted), goes
+ * through a pinned staging array that the batch then keeps (72 bytes per node of
+ * its largest channel). */
 clb_status clb_batch_get_state(clb_batch* b, int k, double* host_f);
 clb_status clb_batch_set_state(clb_batch* b, int k, const double* host_f);
 

@@ -356,8 +356,9 @@ struct clb_batch {
     KC<double>* dkd = nullptr;
     pr::Const* dkp = nullptr;
     double* dobs = nullptr;
-    double* stage = nullptr;      // pinned: one channel's populations in FP64
+    double* stage = nullptr;      // pinned: one channel's populations in FP64 (batch_copy)
     double* stage_dev = nullptr;  // its device address
+    int copies = 0;               // channel states copied before it was made
     double g = 0, ref0 = 0, rho0 = 1, r = 0;
     int64_t step = 0;
     cudaStream_t stream = nullptr;
@@ -676,20 +677,18 @@ clb_status clb_batch_create(int n, const int* nx, const int* ny, const double* k
     b->dch = static_cast<BatchChannel*>(b->dalloc(n * sizeof(BatchChannel)));
     b->dkf = static_cast<KC<float>*>(b->dalloc(n * sizeof(KC<float>)));
     b->dkd = static_cast<KC<double>*>(b->dalloc(n * sizeof(KC<double>)));
-    b->dkp = static_cast<pr::Const*>(b->dalloc(n * sizeof(pr::Const)));
+    const bool f64 = b->storage == CLB_FP64;  // only FP64 collides in pairs
+    if (f64) b->dkp = static_cast<pr::Const*>(b->dalloc(n * sizeof(pr::Const)));
     b->dobs = static_cast<double*>(b->dalloc(9 * (size_t)n * sizeof(double)));
-    if (cudaHostAlloc(reinterpret_cast<void**>(&b->stage), 9 * (size_t)max_nodes * sizeof(double), cudaHostAllocMapped) !=
-            cudaSuccess ||
-        cudaHostGetDevicePointer(reinterpret_cast<void**>(&b->stage_dev), b->stage, 0) != cudaSuccess)
-        cudaGetLastError();
-    if (!b->stage_dev || !b->state || !b->dch || !b->dkf || !b->dkd || !b->dkp || !b->dobs) {
+    if (!b->state || !b->dch || !b->dkf || !b->dkd || (f64 && !b->dkp) || !b->dobs) {
         clb_batch_destroy(b);
         return (clb_status)set_error(CLB_ENOMEM, "clb_batch_create: device allocation failed");
     }
     cudaError_t e = cudaMemcpyAsync(b->dch, b->hch.data(), n * sizeof(BatchChannel), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dkf, kf.data(), n * sizeof(KC<float>), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->dkd, kd.data(), n * sizeof(KC<double>), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dkp, kp.data(), n * sizeof(pr::Const), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && f64)
+        e = cudaMemcpyAsync(b->dkp, kp.data(), n * sizeof(pr::Const), cudaMemcpyHostToDevice, b->stream);
     // initial state f^eq(rho_out, 0) = w_i rho_out: zero deviations (FP32) or w_i rho_out (FP64)
     if (e == cudaSuccess) e = cudaMemsetAsync(b->state, 0, b->total * elem, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -872,26 +871,50 @@ clb_status clb_batch_observables(clb_batch* b, clb_scalars* s) {
     return CLB_OK;
 }
 
-// Channel k's populations to or from a host array: the conversion kernel reads
-// or writes the batch's pinned staging array itself (a transient device buffer
-// and a pageable copy took 21 us per call from Python for 4 x 16 to 4 x 128
-// nodes; this takes 15).
+// Channel k's populations to or from a host array, through a transient device
+// buffer and a pageable copy (21 us per call from Python for 4 x 16 to 4 x 128
+// nodes), or by the conversion kernel from or to the batch's pinned staging array
+// (15 us).  The array takes 350 us to allocate, 58 calls' difference, so it is
+// made once that many calls have been made or, at one for each channel, are to
+// be expected.
+constexpr int kStageCopies = 58;
+
 static clb_status batch_copy(clb_batch* b, int k, double* host, int to_host) {
     if (!b || !host || k < 0 || k >= b->n) return (clb_status)set_error(CLB_EINVAL, "clb_batch state: bad arguments");
     const int nn = b->nx[k] * b->ny[k];
     const long long n = 9LL * nn;
-    if (!to_host) std::memcpy(b->stage, host, n * sizeof(double));
-    const int grid = (int)((n + 255) / 256);
-    if (b->storage == CLB_FP64)
-        batch_canon_kernel<double><<<grid, 256, 0, b->stream>>>(b->state, b->hch[k].offset, n, b->stage_dev, b->ref0,
-                                                                to_host, nn);
-    else
-        batch_canon_kernel<float><<<grid, 256, 0, b->stream>>>(b->state, b->hch[k].offset, n, b->stage_dev, b->ref0,
-                                                               to_host, nn);
-    cudaError_t e = cudaGetLastError();
+    if (!b->stage_dev && b->copies <= kStageCopies && ++b->copies + b->n > kStageCopies) {
+        b->copies = kStageCopies + 1;  // asked for once
+        if (cudaHostAlloc(reinterpret_cast<void**>(&b->stage), 9 * (size_t)b->max_nodes * sizeof(double),
+                          cudaHostAllocMapped) != cudaSuccess ||
+            cudaHostGetDevicePointer(reinterpret_cast<void**>(&b->stage_dev), b->stage, 0) != cudaSuccess)
+            cudaGetLastError();  // the device buffer does without
+    }
+    double* dev = b->stage_dev;
+    if (!dev) dev = static_cast<double*>(b->dalloc(n * sizeof(double)));
+    if (!dev) return (clb_status)set_error(CLB_ENOMEM, "clb_batch state: device allocation failed");
+    const bool staged = dev == b->stage_dev;
+    cudaError_t e = cudaSuccess;
+    if (!to_host) {
+        if (staged)
+            std::memcpy(b->stage, host, n * sizeof(double));
+        else
+            e = cudaMemcpyAsync(dev, host, n * sizeof(double), cudaMemcpyHostToDevice, b->stream);
+    }
+    if (e == cudaSuccess) {
+        const int grid = (int)((n + 255) / 256);
+        if (b->storage == CLB_FP64)
+            batch_canon_kernel<double><<<grid, 256, 0, b->stream>>>(b->state, b->hch[k].offset, n, dev, b->ref0, to_host, nn);
+        else
+            batch_canon_kernel<float><<<grid, 256, 0, b->stream>>>(b->state, b->hch[k].offset, n, dev, b->ref0, to_host, nn);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess && to_host && !staged)
+        e = cudaMemcpyAsync(host, dev, n * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (!staged) b->dfree(dev);
     if (e != cudaSuccess) return (clb_status)set_error(CLB_ECUDA, "clb_batch state: %s", cudaGetErrorString(e));
-    if (to_host) std::memcpy(host, b->stage, n * sizeof(double));
+    if (to_host && staged) std::memcpy(host, b->stage, n * sizeof(double));
     return CLB_OK;
 }
 
