@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_final_kernel(const R* f, R* l
 // step, with a cluster barrier between steps: the states in the blocks' shared
 // memory where each thread has one node (adj_share_*_kernel), in L2 where there
 // are more (adj_cl_*_kernel).
-// 4 x 64 nodes, FP32, per step: forward 0.34 us, backward 0.77 us (0.63 and
+// 4 x 64 nodes, FP32, per step: forward 0.32 us, backward 0.79 us (0.63 and
 // 6.46 us with the pulls worked out every step and J_C^T lambda formed by eleven
 // forward-mode columns over 16 blocks); both are bound by issue and latency in
 // their one block.  A backward step of one warp per scheduler takes 0.58 us

@@ -14,7 +14,7 @@
 // collision instead.  Up to that bound the populations' rms error stays below the
 // plain collision's; at twice the bound it would not (see below).
 //
-// Measured, 25601 x 256 pressure channel: 316 us per sweep against 1455 us;
+// Measured, 25601 x 256 pressure channel: 313 us per sweep against 1455 us;
 // the 18 FP64 operations alone take 225 us.  rms error of a population after
 // one collision, relative to the density, against long double: 8e-18 to 1.6e-17
 // for velocities of 1e-3 to 0.04 and 2.8e-17 at 0.08, against 3.4e-17 of the plain
