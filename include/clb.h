@@ -150,8 +150,10 @@ clb_status clb_create(int nx, int ny, double kn, double a, double r, clb_drive d
                       double drive_value, const clb_opts* opts, clb_sim** out);
 
 /* Advance n >= 0 time steps (Eq. 4-5 with the boundaries above).  Queued on
- * the stream, returns without waiting.  Errors: CLB_EINVAL (n < 0, sim NULL),
- * CLB_ECUDA (launch failure). */
+ * the stream, returns without waiting.  Captured by the caller (calls that replay
+ * no chunk of their own, opts->graph_steps), an even number of steps ends on the
+ * buffer it started from, so that each replay advances the channel by n.
+ * Errors: CLB_EINVAL (n < 0, sim NULL), CLB_ECUDA (launch failure). */
 clb_status clb_step(clb_sim* sim, int64_t n);
 
 /* Scalars of the current state.  Densities and velocities are taken per node

@@ -868,12 +868,13 @@ static cudaError_t launch_single(clb_sim* s, SweepArgs& a, int mode, int cur, in
 }
 
 // Queue n steps from buffer *cur as launches of about equal length, each of at
-// most the steps the engine takes at once; `even`: an even number of launches,
-// so that they end on the buffer they started from.  *done counts the steps queued.
-static cudaError_t launch_steps(clb_sim* s, SweepArgs& a, int mode, int* cur, int64_t n, bool even, int64_t* done) {
+// most the steps the engine takes at once; `parity`: as many launches, odd or
+// even, as steps, so that they end on the buffer that single steps would end on.
+// *done counts the steps queued.
+static cudaError_t launch_steps(clb_sim* s, SweepArgs& a, int mode, int* cur, int64_t n, bool parity, int64_t* done) {
     const int64_t most = s->tile.h > 0 ? s->tile.h : s->march_sms ? 2 : 1;
     int64_t launches = (n + most - 1) / most;
-    if (even && launches % 2) ++launches;
+    if (parity && (launches ^ n) & 1) ++launches;
     *done = 0;
     for (; launches > 0; --launches) {
         int64_t k = (n - *done + launches - 1) / launches;
@@ -926,8 +927,14 @@ clb_status clb_step(clb_sim* s, int64_t n) {
         if (e != cudaSuccess) return fail(CLB_ECUDA, "clb_step: graph launch: %s", cudaGetErrorString(e));
         s->step += s->graph_steps;
     }
+    // a call that the caller captures is replayed from the buffer it started from:
+    // it keeps the parity of single steps, so that an even number of them advances
+    // the channel with every replay
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaSuccess;
+    if (s->tile.h > 0 || s->march_sms) e = cudaStreamIsCapturing(s->stream, &capture);
     int64_t done = 0;
-    const cudaError_t e = launch_steps(s, a, mode, &s->cur, n, false, &done);
+    if (e == cudaSuccess) e = launch_steps(s, a, mode, &s->cur, n, capture != cudaStreamCaptureStatusNone, &done);
     s->step += done;
     if (e != cudaSuccess) return fail(CLB_ECUDA, "clb_step: sweep launch: %s", cudaGetErrorString(e));
     return CLB_OK;
